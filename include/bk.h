@@ -221,6 +221,33 @@ bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, i
                           bk_dtype dtype, const bk_opts* opts, bk_stream_t stream);
 
 /*
+ * bk_matern_tile_ws, bk_matern_tile2_ws: bk_matern_tile_ex and bk_matern_tile2
+ * with caller-owned device scratch (256-byte aligned; one workspace must not
+ * serve two calls that can overlap on the GPU), which takes them to their
+ * fastest paths.  Within one call (sigma^2, beta, nu) are fixed, so an entry is
+ * a function of the squared distance alone: with bk_matern_workspace(rows,
+ * cols) bytes, matrices of at least 2^19 entries are written from a table of
+ * that function that the call first builds in the workspace, on `stream`, from
+ * the integral of Sec. IV-B (piecewise polynomials, errors below those of the
+ * per-entry quadrature; entries with x = r / beta outside about [2.5e-4, 90]
+ * and coincident pairs are evaluated directly).  The table is used for the
+ * searched and learned windows of either compute type, 0.02 <= nu <= 10,
+ * 1e-8 <= beta <= 1e8, 1e-20 <= sigma^2 <= 1e20, and without counters,
+ * search_f64 and series_below (options that ask for the per-entry evaluation).
+ * With at least BK_COSH_TABLE_LEN doubles the plain form otherwise keeps its
+ * e^{-2 nu h} table there (as bk_opts.d_cosh_table); d_work == NULL, or less, is
+ * bk_matern_tile_ex or bk_matern_tile2.  No call allocates.
+ */
+size_t bk_matern_workspace(int64_t rows, int64_t cols);
+bk_status bk_matern_tile_ws(const double* locs, int64_t n, double sigma2, double beta, double nu,
+                            void* out, int64_t ld, bk_dtype dtype, const bk_opts* opts,
+                            void* d_work, size_t work_bytes, bk_stream_t stream);
+bk_status bk_matern_tile2_ws(const double* locs1, int64_t m, const double* locs2, int64_t n,
+                             double sigma2, double beta, double nu, void* out, int64_t ld,
+                             bk_dtype dtype, const bk_opts* opts, void* d_work, size_t work_bytes,
+                             bk_stream_t stream);
+
+/*
  * bk_matern_tile_host: the matrix of bk_matern_tile_ex delivered to HOST
  * memory, with the host <-> device transfers inside the call (Sec. III-A,
  * Algorithm 3; the paper's matrices are consumed by a host-side runtime).
@@ -234,8 +261,8 @@ bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, i
  * cudaHostRegister, and on GB300, whose GPU reaches host page tables through
  * ATS, pageable memory as well), the tile writer stores the matrix straight
  * into h_out over the GPU-CPU link (NVLink-C2C) and d_work needs only
- * bk_matern_tile_host_workspace(n, dtype, 0) bytes (locations and the plain
- * form's e^{-2 nu h} table).  Otherwise, and always with BK_HOST_STAGED,
+ * bk_matern_tile_host_workspace(n, dtype, 0) bytes (locations and the scratch
+ * of bk_matern_tile_ws).  Otherwise, and always with BK_HOST_STAGED,
  * the matrix is staged in d_work, which then needs
  * bk_matern_tile_host_workspace(n, dtype, 1) bytes: it is generated in up to
  * 16 panels of block-columns, and each finished panel's columns are copied to

@@ -35,6 +35,7 @@ BK_TRAIN_TENSOR, BK_TRAIN_SIMT = 0, 1
 EXPORTS = (
     "bk_opts_default", "bk_version", "bk_last_error", "bk_status_string", "bk_sync",
     "bk_eval", "bk_eval_ex", "bk_eval_grad", "bk_eval_autotune", "bk_gaussian_loglik", "bk_matern_tile", "bk_matern_tile_ex", "bk_matern_tile2",
+    "bk_matern_workspace", "bk_matern_tile_ws", "bk_matern_tile2_ws",
     "bk_matern_tile_host", "bk_matern_tile_host_workspace",
     "bk_morton_order", "bk_probe_pipe", "bk_math_probe", "bk_batched_plan_create", "bk_batched_plan_destroy",
     "bk_batched_plan_info", "bk_batched_autotune", "bk_matern_batched",
@@ -97,6 +98,9 @@ def lib() -> ctypes.CDLL:
             "bk_matern_tile": (I, [P, I64, D, D, D, P, I64, I, P]),
             "bk_matern_tile_ex": (I, [P, I64, D, D, D, P, I64, I, P, P]),
             "bk_matern_tile2": (I, [P, I64, P, I64, D, D, D, P, I64, I, P, P]),
+            "bk_matern_workspace": (ctypes.c_size_t, [I64, I64]),
+            "bk_matern_tile_ws": (I, [P, I64, D, D, D, P, I64, I, P, P, ctypes.c_size_t, P]),
+            "bk_matern_tile2_ws": (I, [P, I64, P, I64, D, D, D, P, I64, I, P, P, ctypes.c_size_t, P]),
             "bk_matern_tile_host": (I, [P, I64, D, D, D, P, I64, I, P, I, P, ctypes.c_size_t, P]),
             "bk_matern_tile_host_workspace": (ctypes.c_size_t, [I64, I, I]),
             "bk_morton_order": (I, [P, I64, P]),
@@ -348,25 +352,21 @@ def _locs(locs, name="locs"):
 BK_COSH_TABLE_LEN = 3328
 
 
-def _with_cosh_table(opts, device, dtype_code):
-    """A copy of ``opts`` whose d_cosh_table is a scratch tensor from torch's
-    caching allocator on the current stream (so the library allocates nothing
-    and graph capture takes it from the graph's pool); returns (opts, tensor
-    keeping the scratch alive).  ``opts`` None means the C defaults for a
-    NULL options pointer: default options with compute = the output dtype
-    (FP32 output takes the FP32 precision form)."""
+def _scratch(nbytes: int, device, stream):
+    """Device scratch of ``nbytes`` from torch's caching allocator (so the
+    library allocates nothing and graph capture takes it from the graph's
+    pool).  Freed memory is reused in the order of the current stream; for a
+    call on another stream the allocator is told of that use."""
     torch = _torch()
-    if opts is None:
-        o = bk_opts()
-        lib().bk_opts_default(ctypes.byref(o))
-        o.compute = int(dtype_code)
-    else:
-        o = bk_opts.from_buffer_copy(opts)
-    table = None
-    if not o.d_cosh_table:
-        table = torch.empty(BK_COSH_TABLE_LEN, dtype=torch.float64, device=device)
-        o.d_cosh_table = table.data_ptr()
-    return o, table
+    t = torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device=device)
+    if stream is not None:
+        if isinstance(stream, int):
+            stream = torch.cuda.ExternalStream(stream, device=device) if stream else None
+        if stream is None:
+            stream = torch.cuda.default_stream(device)
+        if stream != torch.cuda.current_stream(device):
+            t.record_stream(stream)
+    return t
 
 
 def bk_matern_tile(locs, sigma2: float, beta: float, nu: float, out=None, dtype=None,
@@ -383,10 +383,10 @@ def bk_matern_tile(locs, sigma2: float, beta: float, nu: float, out=None, dtype=
     if out.dim() != 2 or out.shape[0] != n or out.shape[1] < n:
         raise ValueError("out must be (n, ld) with ld >= n")
     ld = out.shape[1]
-    o, table = _with_cosh_table(opts, locs.device, code)
-    _check(lib().bk_matern_tile_ex(_ptr(locs), n, float(sigma2), float(beta), float(nu), _ptr(out),
-                                   ld, code, ctypes.byref(o), _stream_ptr(stream)))
-    del table  # stream-ordered reuse by torch's allocator is safe after the launch
+    optp = ctypes.byref(opts) if opts is not None else None
+    work = _scratch(lib().bk_matern_workspace(n, n), locs.device, stream)
+    _check(lib().bk_matern_tile_ws(_ptr(locs), n, float(sigma2), float(beta), float(nu), _ptr(out),
+                                   ld, code, optp, _ptr(work), work.numel(), _stream_ptr(stream)))
     return out
 
 
@@ -446,10 +446,11 @@ def bk_matern_tile2(locs1, locs2, sigma2: float, beta: float, nu: float, out=Non
     _dev(out, "out")
     if out.dim() != 2 or out.shape[0] != n or out.shape[1] < m:
         raise ValueError("out must be (n, ld) with ld >= m")
-    o, table = _with_cosh_table(opts, locs1.device, code)
-    _check(lib().bk_matern_tile2(_ptr(locs1), m, _ptr(locs2), n, float(sigma2), float(beta),
-                                 float(nu), _ptr(out), out.shape[1], code, ctypes.byref(o),
-                                 _stream_ptr(stream)))
+    optp = ctypes.byref(opts) if opts is not None else None
+    work = _scratch(lib().bk_matern_workspace(m, n), locs1.device, stream)
+    _check(lib().bk_matern_tile2_ws(_ptr(locs1), m, _ptr(locs2), n, float(sigma2), float(beta),
+                                    float(nu), _ptr(out), out.shape[1], code, optp, _ptr(work),
+                                    work.numel(), _stream_ptr(stream)))
     return out
 
 

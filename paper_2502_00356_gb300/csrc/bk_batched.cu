@@ -25,17 +25,6 @@
 
 namespace bk {
 
-// Work item w (a global tile number) -> instance k with prefix[k] <= w < prefix[k+1].
-__device__ __forceinline__ int find_instance(const int64_t* __restrict__ prefix, int count,
-                                             int64_t w) {
-  int lo = 0, hi = count - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(prefix + mid) <= w) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 template <typename OutT>
 struct BatchSmem {
   SymTileSmem<OutT> tile;
@@ -133,6 +122,8 @@ struct bk_plan {
   int64_t* d_sizes;                // count instance sizes (device)
   unsigned long long* d_next;      // tile counter (device scratch)
   double* d_wnu;                   // count x kCoshTabSize: e^{-2 nu h} per instance, or null
+  void* d_inst;                    // with entry tables: the instances' constants, else null
+  void* d_tables;                  // their tables
   int warps, ctas_per_sm, chunk;   // launch shape
   int tuned;                       // 1 when the shape came from the autotuner or its cache
   double tuned_ms;
@@ -178,8 +169,15 @@ cudaError_t launch_batched_w(const bk_plan* p, const bk_matern_desc* d, int64_t 
   return launch_batched_t<Form, OutT, 8>(p, d, limit, ctas_per_sm, chunk, s);
 }
 
+// FP32 records: FP32 arithmetic into FP32 matrices.
+bool plan_table_f32(const bk_plan* p) { return p->opts.compute == BK_F32 && p->dtype == BK_F32; }
+
 cudaError_t launch_batched(const bk_plan* p, const bk_matern_desc* d, int64_t limit, int warps,
                            int ctas_per_sm, int chunk, cudaStream_t s) {
+  if (p->d_tables != nullptr) {
+    const BatchTable b{p->count, p->d_prefix, p->d_sizes, p->d_next, p->d_inst, p->d_tables};
+    return launch_batched_table(b, d, plan_table_f32(p), p->dtype, limit, warps, ctas_per_sm, chunk, s);
+  }
   cudaError_t e = cudaMemsetAsync(p->d_next, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
   if (p->d_wnu != nullptr) {
@@ -209,6 +207,7 @@ cudaError_t launch_batched(const bk_plan* p, const bk_matern_desc* d, int64_t li
 }
 
 int max_ctas_per_sm(const bk_plan* p, int warps) {
+  if (p->d_tables != nullptr) return batched_table_max_ctas(plan_table_f32(p), p->dtype, warps);
   int blocks = 0;
   const void* fn = nullptr;
   const bool f64 = (p->opts.compute == BK_F64);
@@ -312,8 +311,9 @@ std::string make_key(const bk_plan* p) {
   int bucket = 0;
   while ((1LL << bucket) < p->total_tiles) ++bucket;
   char buf[256];
-  std::snprintf(buf, sizeof(buf), "%s|out%d|compute%d|win%d|tiles2^%d", name.c_str(),
-                (int)p->dtype, (int)p->opts.compute, (int)p->opts.window, bucket);
+  std::snprintf(buf, sizeof(buf), "%s|out%d|compute%d|win%d|tiles2^%d%s", name.c_str(),
+                (int)p->dtype, (int)p->opts.compute, (int)p->opts.window, bucket,
+                p->d_tables != nullptr ? "|table" : "");
   return std::string(buf);
 }
 
@@ -337,10 +337,30 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   if (opts != nullptr) o = *opts; else o.compute = dtype;
   const bk_status st = check_opts(&o);
   if (st != BK_OK) return st;
-  std::vector<int64_t> prefix((size_t)count + 1, 0);
+  // Entry tables (bk_entry_table.cuh) for the forms that have them, when some
+  // instance is worth one and they fit 1 GiB; the others then run in the same
+  // launch without.  The parameters are only known at each call.
+  bool pays = false;
   for (int32_t k = 0; k < count; ++k) {
     if (sizes[k] < 0) return set_error(BK_ERR_INVALID_ARG, "sizes[%d] < 0", (int)k);
-    const int64_t nb = (sizes[k] + kTile - 1) / kTile;
+    pays = pays || entry_table_pays(sizes[k], sizes[k]);
+  }
+  const size_t table_bytes =
+      (size_t)count * entry_table_bytes(o.compute == BK_F32 && dtype == BK_F32);
+  void *d_inst = nullptr, *d_tables = nullptr;
+  if (pays && count <= 65535 && table_bytes <= ((size_t)1 << 30) &&
+      entry_table_applies(o, 1.0, 1.0, 1.0)) {
+    if (cudaMalloc(&d_inst, (size_t)count * batched_instance_bytes()) != cudaSuccess ||
+        cudaMalloc(&d_tables, table_bytes) != cudaSuccess) {
+      (void)cudaGetLastError();  // without them the kernel evaluates every entry itself
+      cudaFree(d_inst);
+      d_inst = d_tables = nullptr;
+    }
+  }
+  const int64_t edge = d_tables != nullptr ? 64 : kTile;
+  std::vector<int64_t> prefix((size_t)count + 1, 0);
+  for (int32_t k = 0; k < count; ++k) {
+    const int64_t nb = (sizes[k] + edge - 1) / edge;
     prefix[(size_t)k + 1] = prefix[(size_t)k] + nb * (nb + 1) / 2;
   }
   bk_plan* p = new bk_plan();
@@ -352,6 +372,8 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   p->d_sizes = nullptr;
   p->d_next = nullptr;
   p->d_wnu = nullptr;
+  p->d_inst = d_inst;
+  p->d_tables = d_tables;
   p->warps = 8;
   p->chunk = 1;
   p->tuned = 0;
@@ -368,7 +390,7 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   // per-instance tables of e^{-2 nu h} for the searched-window FP64 forms
   // (without them, or for more than 4,096 instances, the kernel computes the
   // values itself)
-  if (e == cudaSuccess && o.compute == BK_F64 && o.window != BK_WIN_FIXED &&
+  if (e == cudaSuccess && d_tables == nullptr && o.compute == BK_F64 && o.window != BK_WIN_FIXED &&
       o.window != BK_WIN_LEARNED && count <= 4096) {
     if (cudaMalloc((void**)&p->d_wnu, (size_t)count * kCoshTabSize * sizeof(double)) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -379,11 +401,13 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
     cudaFree(p->d_prefix);
     cudaFree(p->d_sizes);
     cudaFree(p->d_next);
+    cudaFree(p->d_inst);
+    cudaFree(p->d_tables);
     delete p;
     return (e == cudaErrorMemoryAllocation) ? set_error(BK_ERR_NOMEM, "plan: out of device memory")
                                             : check_cuda(e, "bk_batched_plan_create");
   }
-  p->ctas_per_sm = std::min(2, max_ctas_per_sm(p, p->warps));
+  p->ctas_per_sm = std::min(p->d_tables != nullptr ? 4 : 2, max_ctas_per_sm(p, p->warps));
   p->key = make_key(p);
   int w, c, ch;
   double ms;
@@ -405,6 +429,8 @@ bk_status bk_batched_plan_destroy(bk_plan* plan) {
   cudaFree(plan->d_sizes);
   cudaFree(plan->d_next);
   cudaFree(plan->d_wnu);
+  cudaFree(plan->d_inst);
+  cudaFree(plan->d_tables);
   delete plan;
   return BK_OK;
 }

@@ -126,7 +126,29 @@ bk_status check_matrix(const void* out, int64_t rows, int64_t cols, int64_t ld) 
   return BK_OK;
 }
 
+bk_status check_work(const void* d_work) {
+  if (((uintptr_t)d_work & 255) != 0)
+    return set_error(BK_ERR_INVALID_ARG, "d_work must be 256-byte aligned");
+  return BK_OK;
+}
+
 }  // namespace
+
+size_t matern_scratch_bytes(bool table) {
+  return kEntryTableOffset + (table ? std::max(entry_table_bytes(false), entry_table_bytes(true)) : 0);
+}
+
+void* matern_scratch(bk_opts& o, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
+                     void* d_work, size_t work_bytes) {
+  if (d_work == nullptr) return nullptr;
+  if (entry_table_pays(rows, cols) && work_bytes >= matern_scratch_bytes(true) &&
+      entry_table_applies(o, sigma2, beta, nu))
+    return (char*)d_work + kEntryTableOffset;
+  if (o.compute == BK_F64 && o.d_cosh_table == nullptr && work_bytes >= kEntryTableOffset)
+    o.d_cosh_table = (double*)d_work;
+  return nullptr;
+}
+
 }  // namespace bk
 
 using namespace bk;
@@ -290,9 +312,13 @@ bk_status bk_eval(const double* x, const double* nu, double* out, int64_t n, bk_
   return bk_eval_ex(x, nu, out, nullptr, BK_F64, n, nullptr, stream);
 }
 
-bk_status bk_matern_tile_ex(const double* locs, int64_t n, double sigma2, double beta, double nu,
+size_t bk_matern_workspace(int64_t rows, int64_t cols) {
+  return matern_scratch_bytes(entry_table_pays(rows, cols));
+}
+
+bk_status bk_matern_tile_ws(const double* locs, int64_t n, double sigma2, double beta, double nu,
                             void* out, int64_t ld, bk_dtype dtype, const bk_opts* opts,
-                            bk_stream_t stream) {
+                            void* d_work, size_t work_bytes, bk_stream_t stream) {
   bk_opts o;
   bk_opts_default(&o);
   if (opts != nullptr) o = *opts;
@@ -302,11 +328,15 @@ bk_status bk_matern_tile_ex(const double* locs, int64_t n, double sigma2, double
   if ((st = check_matrix(out, n, n, ld)) != BK_OK) return st;
   if (opts == nullptr) o.compute = dtype;  // the output dtype picks the form by default
   if ((st = check_opts(&o)) != BK_OK) return st;
+  if ((st = check_work(d_work)) != BK_OK) return st;
   if (n == 0) return BK_OK;
   if (locs == nullptr) return set_error(BK_ERR_INVALID_ARG, "locs is NULL");
   cudaStream_t s = (cudaStream_t)stream;
+  void* const table = matern_scratch(o, n, n, sigma2, beta, nu, d_work, work_bytes);
   const cudaError_t e =
-      (o.window == BK_WIN_LEARNED)
+      (table != nullptr)
+          ? launch_matern_sym_table(locs, n, sigma2, beta, nu, out, ld, dtype, o.compute, table, s)
+      : (o.window == BK_WIN_LEARNED)
           ? launch_matern_sym_learned(o.learned, locs, n, sigma2, beta, nu, out, ld, dtype,
                                       o.d_counters, s)
       : (o.compute == BK_F64)
@@ -315,14 +345,21 @@ bk_status bk_matern_tile_ex(const double* locs, int64_t n, double sigma2, double
   return check_cuda(e, "bk_matern_tile launch");
 }
 
+bk_status bk_matern_tile_ex(const double* locs, int64_t n, double sigma2, double beta, double nu,
+                            void* out, int64_t ld, bk_dtype dtype, const bk_opts* opts,
+                            bk_stream_t stream) {
+  return bk_matern_tile_ws(locs, n, sigma2, beta, nu, out, ld, dtype, opts, nullptr, 0, stream);
+}
+
 bk_status bk_matern_tile(const double* locs, int64_t n, double sigma2, double beta, double nu,
                          void* out, int64_t ld, bk_dtype dtype, bk_stream_t stream) {
   return bk_matern_tile_ex(locs, n, sigma2, beta, nu, out, ld, dtype, nullptr, stream);
 }
 
-bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, int64_t n,
-                          double sigma2, double beta, double nu, void* out, int64_t ld,
-                          bk_dtype dtype, const bk_opts* opts, bk_stream_t stream) {
+bk_status bk_matern_tile2_ws(const double* locs1, int64_t m, const double* locs2, int64_t n,
+                             double sigma2, double beta, double nu, void* out, int64_t ld,
+                             bk_dtype dtype, const bk_opts* opts, void* d_work, size_t work_bytes,
+                             bk_stream_t stream) {
   bk_opts o;
   bk_opts_default(&o);
   bk_status st;
@@ -331,12 +368,17 @@ bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, i
   if ((st = check_theta(sigma2, beta, nu)) != BK_OK) return st;
   if ((st = check_matrix(out, m, n, ld)) != BK_OK) return st;
   if ((st = check_opts(&o)) != BK_OK) return st;
+  if ((st = check_work(d_work)) != BK_OK) return st;
   if (m == 0 || n == 0) return BK_OK;
   if (locs1 == nullptr || locs2 == nullptr)
     return set_error(BK_ERR_INVALID_ARG, "locs1 and locs2 must be non-NULL");
   cudaStream_t s = (cudaStream_t)stream;
+  void* const table = matern_scratch(o, m, n, sigma2, beta, nu, d_work, work_bytes);
   const cudaError_t e =
-      (o.window == BK_WIN_LEARNED)
+      (table != nullptr)
+          ? launch_matern_block_table(locs1, m, locs2, n, sigma2, beta, nu, out, ld, dtype,
+                                      o.compute, table, s)
+      : (o.window == BK_WIN_LEARNED)
           ? launch_matern_block_learned(o.learned, locs1, m, locs2, n, sigma2, beta, nu, out, ld,
                                         dtype, o.d_counters, s)
       : (o.compute == BK_F64)
@@ -345,6 +387,13 @@ bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, i
           : launch_matern_block_f32(locs1, m, locs2, n, sigma2, beta, nu, out, ld, dtype,
                                     o.d_counters, s);
   return check_cuda(e, "bk_matern_tile2 launch");
+}
+
+bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, int64_t n,
+                          double sigma2, double beta, double nu, void* out, int64_t ld,
+                          bk_dtype dtype, const bk_opts* opts, bk_stream_t stream) {
+  return bk_matern_tile2_ws(locs1, m, locs2, n, sigma2, beta, nu, out, ld, dtype, opts, nullptr, 0,
+                            stream);
 }
 
 bk_status bk_morton_order(const double* locs, int64_t n, int64_t* perm) {

@@ -1,0 +1,269 @@
+// The Matern tile writers that evaluate their entries from a per-call table
+// (bk_entry_table.cuh): the table's kernel, the symmetric writer and the m x n
+// block writer, and the rule that takes a call to them.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "bk_entry_table.cuh"
+#include "bk_internal.h"
+#include "bk_tiles.cuh"
+
+namespace bk {
+namespace {
+
+// The table of one call.  Up to kTabScan locations, every block first bounds
+// the distances (1.5 us there), and the binades beyond the bound are left out:
+// for x up to 14 that is two thirds of the intervals.
+constexpr int64_t kTabScan = 8192;
+template <bool F32>
+__global__ void __launch_bounds__(kTabThreads) entry_table_kernel(
+    const __grid_constant__ MaternParams mp, const double* __restrict__ locs1, int64_t m,
+    const double* __restrict__ locs2, int64_t n, unsigned char* __restrict__ table) {
+  __shared__ TabBuildSmem sm;
+  const double r2_max = m + n <= 2 * kTabScan ? tab_r2_bound(sm.box, locs1, m, locs2, n) : kInf;
+  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, r2_max, table);
+}
+
+// One 64 x 64 tile per block of 256 threads; lane i of warp w evaluates rows
+// i and i + 32 against columns 8 w .. 8 w + 7.  Block (I, J) is stored straight
+// from registers (a warp writes 32 consecutive rows of one column); for a
+// symmetric matrix the tile also goes through shared memory to block (J, I).
+// col_base as in matern_sym_kernel, in tiles of 64.
+template <bool F32, typename OutT, bool kSym>
+__global__ void __launch_bounds__(256, 4) matern_table_kernel(
+    const unsigned char* __restrict__ table, const double* __restrict__ locs1, int64_t m,
+    const double* __restrict__ locs2, int64_t n, const __grid_constant__ MaternParams mp,
+    OutT* __restrict__ out, int64_t ld, int64_t tiles_m, int64_t col_base, int width) {
+  __shared__ TabTileSmem<OutT> sm;
+  const unsigned e0 = tab_first_binade(mp.inv_beta);
+  tab_stage_octaves<F32>(sm.oct, e0);
+  const unsigned parts = kTabTile / width, tile = blockIdx.x / parts, part = blockIdx.x % parts;
+  int64_t I, J;
+  if constexpr (kSym) {
+    if (col_base < 0) tri_tile(tile, I, J);
+    else col_tile(col_base + tile, tiles_m, I, J);
+  } else {
+    I = tile % tiles_m;
+    J = tile / tiles_m;
+  }
+  tab_tile<F32, OutT, kSym, 8>(sm, table, e0, locs1, m, locs2, n, I, J, mp, out, ld, (int)part, width);
+}
+
+// ---- batched: every instance's constants, tables and tiles in three launches
+__global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_desc* __restrict__ descs,
+                                                             const int64_t* __restrict__ sizes,
+                                                             int count, BatchInstance* __restrict__ inst,
+                                                             unsigned long long* __restrict__ next) {
+  const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (k == 0) *next = 0ull;
+  if (k >= count) return;
+  const bk_matern_desc d = descs[k];
+  // a descriptor that does not match the plan is skipped (n = 0)
+  const bool ok = d.n == sizes[k] && d.ld >= d.n && d.locs != nullptr && d.out != nullptr &&
+                  d.beta > 0.0 && d.nu > 0.0 && d.sigma2 >= 0.0;
+  BatchInstance b;
+  b.locs = d.locs;
+  b.out = d.out;
+  b.n = ok ? d.n : 0;
+  b.ld = d.ld;
+  b.table = ok && entry_table_size(d.n, d.n) && tab_domain(d.sigma2, d.beta, d.nu);
+  b.mp = matern_params(d.sigma2, d.beta, d.nu);
+  inst[k] = b;
+}
+
+template <bool F32>
+__global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
+    const BatchInstance* __restrict__ inst, unsigned char* __restrict__ tables) {
+  __shared__ TabBuildSmem sm;
+  const BatchInstance& b = inst[blockIdx.y];
+  if (!b.table) return;
+  const MaternParams mp = b.mp;
+  const double r2_max = b.n <= kTabScan ? tab_r2_bound(sm.box, b.locs, b.n, b.locs, b.n) : kInf;
+  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, r2_max,
+                       tables + (size_t)blockIdx.y * TabLayout<F32>::kBytes);
+}
+
+// Persistent kernel as matern_batched_kernel, in tiles of 64.
+template <bool F32, typename OutT, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_kernel(
+    const BatchInstance* __restrict__ inst, int count, const int64_t* __restrict__ prefix,
+    int64_t limit, unsigned long long* __restrict__ next, int chunk,
+    const unsigned char* __restrict__ tables) {
+  __shared__ TabTileSmem<OutT> sm;
+  __shared__ BatchInstance cur;
+  __shared__ int64_t item;
+  int k = -1;
+  while (true) {
+    __syncthreads();  // shared data of the previous round is no longer read
+    if (threadIdx.x == 0) item = (int64_t)atomicAdd(next, (unsigned long long)chunk);
+    __syncthreads();
+    const int64_t base = item;
+    if (base >= limit) break;
+    const int64_t end = min(base + (int64_t)chunk, limit);
+    for (int64_t w = base; w < end; ++w) {
+      const int kw = find_instance(prefix, count, w);
+      __syncthreads();
+      if (kw != k) {
+        k = kw;
+        constexpr int kWords = (int)(sizeof(BatchInstance) / 8);
+        static_assert(sizeof(BatchInstance) % 8 == 0 && kWords <= 128, "copied by the block's threads");
+        if (threadIdx.x < kWords)
+          reinterpret_cast<long long*>(&cur)[threadIdx.x] =
+              reinterpret_cast<const long long*>(inst + k)[threadIdx.x];
+        __syncthreads();
+        tab_stage_octaves<F32>(sm.oct, tab_first_binade(cur.mp.inv_beta));
+      }
+      int64_t I, J;
+      tri_tile(w - __ldg(prefix + k), I, J);
+      tab_tile<F32, OutT, true, WARPS>(sm, tables + (size_t)k * TabLayout<F32>::kBytes,
+                                       tab_first_binade(cur.mp.inv_beta), cur.locs, cur.n, cur.locs,
+                                       cur.n, I, J, cur.mp, (OutT*)cur.out, cur.ld, 0, kTabTile,
+                                       cur.table != 0);
+    }
+  }
+}
+
+}  // namespace
+
+size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kBytes : TabLayout64::kBytes; }
+
+// entry_table_size (the header): from 2^19 entries on (n = 725) a matrix is worth a table.  The table itself
+// costs about 5 us (its kernel and the launch), what the direct evaluation
+// takes for 2^16 entries; between the two, small matrices keep the direct
+// path, whose results do not depend on whether the caller has scratch memory.
+bool entry_table_pays(int64_t rows, int64_t cols) { return entry_table_size(rows, cols); }
+
+bool entry_table_applies(const bk_opts& o, double sigma2, double beta, double nu) {
+  return o.d_counters == nullptr && o.window != BK_WIN_FIXED && o.series_below == 0.0 &&
+         o.search_f64 == 0 && tab_domain(sigma2, beta, nu);
+}
+
+namespace {
+
+// Whole tiles where they fill the SMs' four slots once, else quarters of 16
+// columns (n = 777: 91 tiles on 152 SMs, 14.8 us whole).
+int tile_width(int64_t ntiles) {
+  return ntiles < (int64_t)current_sm_count() * 4 ? kTabTile / 4 : kTabTile;
+}
+
+template <bool F32>
+cudaError_t build_table(const MaternParams& mp, const double* locs1, int64_t m,
+                        const double* locs2, int64_t n, unsigned char* table, cudaStream_t s) {
+  constexpr int grid = (TabLayout<F32>::kBins + kTabBinsPerBlock - 1) / kTabBinsPerBlock;
+  entry_table_kernel<F32><<<grid, kTabThreads, 0, s>>>(mp, locs1, m, locs2, n, table);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_matern_sym_table(const double* locs, int64_t n, double sigma2, double beta,
+                                    double nu, void* out, int64_t ld, bk_dtype out_t,
+                                    bk_dtype compute, void* table, cudaStream_t s,
+                                    const SymRange& range) {
+  const MaternParams mp = matern_params_host(sigma2, beta, nu);
+  unsigned char* const tab = (unsigned char*)table;
+  const bool f32 = compute == BK_F32 && out_t == BK_F32;
+  if (range.fill_table) {
+    const cudaError_t e = f32 ? build_table<true>(mp, locs, n, locs, n, tab, s)
+                              : build_table<false>(mp, locs, n, locs, n, tab, s);
+    if (e != cudaSuccess) return e;
+  }
+  const int64_t nb = (n + kTabTile - 1) / kTabTile;
+  int64_t ntiles = nb * (nb + 1) / 2, col_base = -1;
+  if (range.j1 >= 0) {
+    const int64_t j0 = range.j0 < 0 ? 0 : range.j0, j1 = range.j1 < nb ? range.j1 : nb;
+    if (j1 <= j0) return cudaSuccess;
+    col_base = j0 * nb - j0 * (j0 - 1) / 2;
+    ntiles = (j1 * nb - j1 * (j1 - 1) / 2) - col_base;
+  }
+  if (ntiles > 2147483647) return cudaErrorInvalidConfiguration;
+  const int width = tile_width(ntiles);
+  const unsigned grid = (unsigned)(ntiles * (kTabTile / width));
+  if (f32)
+    matern_table_kernel<true, float, true><<<grid, 256, 0, s>>>(tab, locs, n, locs, n, mp, (float*)out,
+                                                                ld, nb, col_base, width);
+  else if (out_t == BK_F32)
+    matern_table_kernel<false, float, true><<<grid, 256, 0, s>>>(tab, locs, n, locs, n, mp,
+                                                                 (float*)out, ld, nb, col_base, width);
+  else
+    matern_table_kernel<false, double, true><<<grid, 256, 0, s>>>(tab, locs, n, locs, n, mp,
+                                                                  (double*)out, ld, nb, col_base, width);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_matern_block_table(const double* locs1, int64_t m, const double* locs2, int64_t n,
+                                      double sigma2, double beta, double nu, void* out, int64_t ld,
+                                      bk_dtype out_t, bk_dtype compute, void* table, cudaStream_t s) {
+  const MaternParams mp = matern_params_host(sigma2, beta, nu);
+  unsigned char* const tab = (unsigned char*)table;
+  const bool f32 = compute == BK_F32 && out_t == BK_F32;
+  const cudaError_t e = f32 ? build_table<true>(mp, locs1, m, locs2, n, tab, s)
+                            : build_table<false>(mp, locs1, m, locs2, n, tab, s);
+  if (e != cudaSuccess) return e;
+  const int64_t tm = (m + kTabTile - 1) / kTabTile, tn = (n + kTabTile - 1) / kTabTile;
+  if (tm * tn > 2147483647) return cudaErrorInvalidConfiguration;
+  const int width = tile_width(tm * tn);
+  const unsigned grid = (unsigned)(tm * tn * (kTabTile / width));
+  if (f32)
+    matern_table_kernel<true, float, false><<<grid, 256, 0, s>>>(tab, locs1, m, locs2, n, mp,
+                                                                 (float*)out, ld, tm, -1, width);
+  else if (out_t == BK_F32)
+    matern_table_kernel<false, float, false><<<grid, 256, 0, s>>>(tab, locs1, m, locs2, n, mp,
+                                                                  (float*)out, ld, tm, -1, width);
+  else
+    matern_table_kernel<false, double, false><<<grid, 256, 0, s>>>(tab, locs1, m, locs2, n, mp,
+                                                                   (double*)out, ld, tm, -1, width);
+  return cudaGetLastError();
+}
+
+
+size_t batched_instance_bytes() { return sizeof(BatchInstance); }
+
+namespace {
+
+template <bool F32, typename OutT>
+cudaError_t launch_batched_table_t(const BatchTable& b, int64_t limit, int warps, int ctas_per_sm,
+                                   int chunk, cudaStream_t s) {
+  // 16 (4) blocks share an instance's FP64 (FP32) table: the node weights, once
+  // per block, stay a small part of it
+  batched_table_kernel<F32><<<dim3(F32 ? 4 : 16, (unsigned)b.count), kTabThreads, 0, s>>>(
+      (const BatchInstance*)b.instances, (unsigned char*)b.tables);
+  const int grid = current_sm_count() * ctas_per_sm;
+  if (warps == 4)
+    matern_batched_table_kernel<F32, OutT, 4><<<grid, 128, 0, s>>>(
+        (const BatchInstance*)b.instances, b.count, b.prefix, limit, b.next, chunk,
+        (const unsigned char*)b.tables);
+  else
+    matern_batched_table_kernel<F32, OutT, 8><<<grid, 256, 0, s>>>(
+        (const BatchInstance*)b.instances, b.count, b.prefix, limit, b.next, chunk,
+        (const unsigned char*)b.tables);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* descs, bool f32,
+                                 bk_dtype out_t, int64_t limit, int warps, int ctas_per_sm, int chunk,
+                                 cudaStream_t s) {
+  batched_params_kernel<<<(unsigned)((b.count + 127) / 128), 128, 0, s>>>(
+      descs, b.sizes, b.count, (BatchInstance*)b.instances, b.next);
+  if (f32) return launch_batched_table_t<true, float>(b, limit, warps, ctas_per_sm, chunk, s);
+  if (out_t == BK_F32) return launch_batched_table_t<false, float>(b, limit, warps, ctas_per_sm, chunk, s);
+  return launch_batched_table_t<false, double>(b, limit, warps, ctas_per_sm, chunk, s);
+}
+
+int batched_table_max_ctas(bool f32, bk_dtype out_t, int warps) {
+  const void* fn =
+      f32 ? (warps == 4 ? (const void*)matern_batched_table_kernel<true, float, 4>
+                        : (const void*)matern_batched_table_kernel<true, float, 8>)
+      : out_t == BK_F32 ? (warps == 4 ? (const void*)matern_batched_table_kernel<false, float, 4>
+                                      : (const void*)matern_batched_table_kernel<false, float, 8>)
+                        : (warps == 4 ? (const void*)matern_batched_table_kernel<false, double, 4>
+                                      : (const void*)matern_batched_table_kernel<false, double, 8>);
+  int blocks = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, warps * 32, 0) != cudaSuccess) return 1;
+  return blocks < 1 ? 1 : blocks;
+}
+
+}  // namespace bk

@@ -30,21 +30,21 @@ namespace bk {
 namespace {
 
 constexpr int kMaxPanels = 16;
-constexpr int kBlock = 32;
+constexpr int kBlock = 64;  // columns of a panel unit (SymRange)
 constexpr size_t kAlign = 256;
 
 size_t round_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
-// Workspace layout: locations (16 n bytes), the e^{-2 nu h} table of the
-// plain form, then the n x n matrix with leading dimension n.
+// Workspace layout: locations (16 n bytes), the scratch of the tile writers
+// (matern_scratch), then the n x n matrix with leading dimension n.
 struct Layout {
-  size_t locs, table, matrix, total;
+  size_t locs, scratch, matrix, total;
 };
 Layout layout(int64_t n, bk_dtype dtype) {
   Layout L;
   L.locs = 0;
-  L.table = round_up((size_t)n * 2 * sizeof(double));
-  L.matrix = L.table + round_up((size_t)BK_COSH_TABLE_LEN * sizeof(double));
+  L.scratch = round_up((size_t)n * 2 * sizeof(double));
+  L.matrix = L.scratch + round_up(matern_scratch_bytes(entry_table_pays(n, n)));
   const size_t elem = dtype == BK_F64 ? sizeof(double) : sizeof(float);
   L.total = L.matrix + (size_t)n * (size_t)n * elem;
   return L;
@@ -152,12 +152,15 @@ bk_status bk_matern_tile_host(const double* h_locs, int64_t n, double sigma2, do
 
   char* ws = (char*)d_work;
   double* d_locs = (double*)(ws + L.locs);
-  if (o.compute == BK_F64 && o.d_cosh_table == nullptr) o.d_cosh_table = (double*)(ws + L.table);
+  void* const table = matern_scratch(o, n, n, sigma2, beta, nu, ws + L.scratch, L.matrix - L.scratch);
   const size_t elem = dtype == BK_F64 ? sizeof(double) : sizeof(float);
   cudaStream_t s = (cudaStream_t)stream;
 
   auto launch = [&](void* out, int64_t ldo, const SymRange& r) {
-    return (o.window == BK_WIN_LEARNED)
+    return (table != nullptr)
+               ? launch_matern_sym_table(d_locs, n, sigma2, beta, nu, out, ldo, dtype, o.compute,
+                                         table, s, r)
+           : (o.window == BK_WIN_LEARNED)
                ? launch_matern_sym_learned(o.learned, d_locs, n, sigma2, beta, nu, out, ldo, dtype,
                                            o.d_counters, s, r)
            : (o.compute == BK_F64)

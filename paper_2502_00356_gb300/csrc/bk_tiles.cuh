@@ -357,7 +357,9 @@ __device__ __forceinline__ void sym_tile(const Form& form, SymTileSmem<OutT>& sm
 
 // Lower-triangle tile number t = I (I + 1)/2 + J  ->  (I, J).
 __device__ __forceinline__ void tri_tile(int64_t t, int64_t& I, int64_t& J) {
-  I = (int64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+  // an FP32 seed and exact integer steps: an FP64 square root per thread took
+  // the FP64 pipe as long as an eighth of a tile of the plain form
+  I = (int64_t)((sqrtf(fmaf(8.0f, (float)t, 1.0f)) - 1.0f) * 0.5f);
   while (I * (I + 1) / 2 > t) --I;
   while ((I + 1) * (I + 2) / 2 <= t) ++I;
   J = t - I * (I + 1) / 2;
@@ -372,12 +374,23 @@ __device__ __forceinline__ int64_t col_tile_offset(int64_t J, int64_t nb) {
   return J * nb - J * (J - 1) / 2;
 }
 __device__ __forceinline__ void col_tile(int64_t T, int64_t nb, int64_t& I, int64_t& J) {
-  const double b = 2.0 * (double)nb + 1.0;
-  J = (int64_t)(0.5 * (b - sqrt(fmax(b * b - 8.0 * (double)T, 0.0))));
+  const float b = 2.0f * (float)nb + 1.0f;
+  J = (int64_t)(0.5f * (b - sqrtf(fmaxf(fmaf(b, b, -8.0f * (float)T), 0.0f))));
   if (J < 0) J = 0;
   while (J > 0 && col_tile_offset(J, nb) > T) --J;
   while (col_tile_offset(J + 1, nb) <= T) ++J;
   I = J + (T - col_tile_offset(J, nb));
+}
+
+// Work item w (a global tile number) -> instance k with prefix[k] <= w < prefix[k+1].
+__device__ __forceinline__ int find_instance(const int64_t* __restrict__ prefix, int count,
+                                             int64_t w) {
+  int lo = 0, hi = count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(prefix + mid) <= w) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
 
 // Full symmetric matrix: block b computes the lower-triangle tiles
@@ -509,8 +522,8 @@ cudaError_t launch_matern_sym_form(const Form& form, const double* locs, int64_t
   if (n == 0) return cudaSuccess;
   const int64_t nb = (n + kTile - 1) / kTile;
   int64_t ntiles = nb * (nb + 1) / 2, col_base = -1;
-  if (range.j1 >= 0) {  // block-columns [j0, j1) in block-column order
-    const int64_t j0 = range.j0 < 0 ? 0 : range.j0, j1 = range.j1 < nb ? range.j1 : nb;
+  if (range.j1 >= 0) {  // block-columns in block-column order, two tiles to a range unit of 64
+    const int64_t j0 = range.j0 < 0 ? 0 : 2 * range.j0, j1 = 2 * range.j1 < nb ? 2 * range.j1 : nb;
     if (j1 <= j0) return cudaSuccess;
     col_base = j0 * nb - j0 * (j0 - 1) / 2;
     ntiles = (j1 * nb - j1 * (j1 - 1) / 2) - col_base;
