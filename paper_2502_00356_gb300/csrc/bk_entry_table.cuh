@@ -500,13 +500,16 @@ struct TabTileSmem {
   OutT tile[kTabTile][kTabTile + 1];
 };
 
-// A coordinate as two floats (hi + lo) without conversions on the FP64 pipe.
+// A coordinate as two floats (hi + lo) on the integer pipe.  What those do not
+// hold (tiny, huge, not finite) becomes NaN, which no table contains: its
+// entries take the direct evaluation.  (A branch to conversions instead was
+// executed by every thread: 200 FP64-pipe instructions a tile, half its time.)
 __device__ __forceinline__ void split_bits(double v, float& h, float& l) {
   bool ok;
   const DF d = df_from_bits(v, ok);
-  h = d.hi;
-  l = d.lo;
-  if (!ok) split_f(v, h, l);  // zero, tiny, huge, not finite
+  const bool zero = ((__double2hiint(v) << 1) | __double2loint(v)) == 0;
+  h = ok ? d.hi : zero ? 0.0f : __int_as_float(0x7fc00000);
+  l = ok ? d.lo : 0.0f;
 }
 
 // One 64 x 64 tile (I, J) of M between locs1 (rows) and locs2 (columns) by a

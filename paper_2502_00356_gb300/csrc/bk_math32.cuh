@@ -340,7 +340,7 @@ __device__ __forceinline__ DF df_from_bits(double v, bool& ok) {
   const float hi = __int_as_float((int)(sign | ((unsigned)(eh + 127) << 23) | ((unsigned)q & 0x7fffffu)));
   // r 2^(e-52): the exponent can fall below the float range; split the scale
   const int s1 = (e - 52) / 2, s2 = (e - 52) - s1;
-  const float lo = (float)r * __int_as_float((s1 + 127) << 23) * __int_as_float((s2 + 127) << 23);
+  const float lo = (float)(int)r * __int_as_float((s1 + 127) << 23) * __int_as_float((s2 + 127) << 23);
   return DF{hi, __int_as_float(__float_as_int(lo) ^ (int)sign)};
 }
 
