@@ -448,6 +448,21 @@ bk_status bk_matern_batched_static(const bk_matern_desc* d_descs, int32_t count,
 bk_status bk_gaussian_loglik(double* a, int64_t n, int64_t ld, const double* z, double* y,
                              double* out, const bk_opts* opts, bk_stream_t stream);
 
+/* bk_gaussian_loglik_ws: bk_gaussian_loglik with caller-owned device scratch
+ * (256-byte aligned, bk_gaussian_loglik_workspace(n) bytes; one workspace must
+ * not serve two calls that can overlap on the GPU).  The factorisation then runs
+ * in 64-bit fixed point, scaled by powers of two from the diagonal (60 fraction
+ * bits of sqrt(a_ii a_jj)): the trailing updates as exact digit products on the
+ * tensor cores (tcgen05), the panels on the integer pipe.  Its rounding is
+ * below that of FP64 relative to sqrt(a_ii a_jj); entries of L far below their
+ * row's norm carry that absolute accuracy.  A matrix with |a_ij| >= 2
+ * sqrt(a_ii a_jj) or a non-finite entry counts as not positive definite.  Two
+ * launches per 64 rows.  d_work == NULL or too small: bk_gaussian_loglik. */
+size_t bk_gaussian_loglik_workspace(int64_t n);
+bk_status bk_gaussian_loglik_ws(double* a, int64_t n, int64_t ld, const double* z, double* y,
+                                double* out, const bk_opts* opts, void* d_work, size_t work_bytes,
+                                bk_stream_t stream);
+
 /*
  * bk_probe_pipe: throughput probe for the roofline denominators (not part of
  * the paper's method).  Launches grid x block threads; each runs `iters`

@@ -34,7 +34,8 @@ BK_TRAIN_TENSOR, BK_TRAIN_SIMT = 0, 1
 #: every symbol include/bk.h declares (checked by the CPU tests)
 EXPORTS = (
     "bk_opts_default", "bk_version", "bk_last_error", "bk_status_string", "bk_sync",
-    "bk_eval", "bk_eval_ex", "bk_eval_grad", "bk_eval_autotune", "bk_gaussian_loglik", "bk_matern_tile", "bk_matern_tile_ex", "bk_matern_tile2",
+    "bk_eval", "bk_eval_ex", "bk_eval_grad", "bk_eval_autotune", "bk_gaussian_loglik", "bk_gaussian_loglik_workspace",
+    "bk_gaussian_loglik_ws", "bk_matern_tile", "bk_matern_tile_ex", "bk_matern_tile2",
     "bk_matern_workspace", "bk_matern_tile_ws", "bk_matern_tile2_ws",
     "bk_matern_tile_host", "bk_matern_tile_host_workspace",
     "bk_morton_order", "bk_probe_pipe", "bk_math_probe", "bk_batched_plan_create", "bk_batched_plan_destroy",
@@ -95,6 +96,8 @@ def lib() -> ctypes.CDLL:
             "bk_eval_grad": (I, [P, P, P, P, P, I64, P, P]),
             "bk_eval_autotune": (I, [P, P, P, I, I64, P, P, P]),
             "bk_gaussian_loglik": (I, [P, I64, I64, P, P, P, P, P]),
+            "bk_gaussian_loglik_workspace": (ctypes.c_size_t, [I64]),
+            "bk_gaussian_loglik_ws": (I, [P, I64, I64, P, P, P, P, P, ctypes.c_size_t, P]),
             "bk_matern_tile": (I, [P, I64, D, D, D, P, I64, I, P]),
             "bk_matern_tile_ex": (I, [P, I64, D, D, D, P, I64, I, P, P]),
             "bk_matern_tile2": (I, [P, I64, P, I64, D, D, D, P, I64, I, P, P]),
@@ -336,8 +339,9 @@ def bk_gaussian_loglik(a, z, y=None, out=None, opts: Optional[bk_opts] = None, s
     _dev(y, "y", torch.float64)
     _dev(out, "out", torch.float64)
     optp = ctypes.byref(opts) if opts is not None else None
-    _check(lib().bk_gaussian_loglik(_ptr(a), n, ld, _ptr(z), _ptr(y), _ptr(out), optp,
-                                    _stream_ptr(stream)))
+    work = _scratch(lib().bk_gaussian_loglik_workspace(n), a.device, stream)
+    _check(lib().bk_gaussian_loglik_ws(_ptr(a), n, ld, _ptr(z), _ptr(y), _ptr(out), optp, _ptr(work),
+                                       work.numel(), _stream_ptr(stream)))
     return out
 
 

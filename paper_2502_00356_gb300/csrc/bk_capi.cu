@@ -288,8 +288,11 @@ bk_status bk_eval_grad(const double* x, const double* nu, double* k, double* dk_
                     "bk_eval_grad launch");
 }
 
-bk_status bk_gaussian_loglik(double* a, int64_t n, int64_t ld, const double* z, double* y,
-                             double* out, const bk_opts* opts, bk_stream_t stream) {
+size_t bk_gaussian_loglik_workspace(int64_t n) { return n > 0 ? loglik_workspace_bytes(n) : 0; }
+
+bk_status bk_gaussian_loglik_ws(double* a, int64_t n, int64_t ld, const double* z, double* y,
+                                double* out, const bk_opts* opts, void* d_work, size_t work_bytes,
+                                bk_stream_t stream) {
   bk_opts o;
   bk_opts_default(&o);
   if (opts != nullptr) o = *opts;
@@ -305,7 +308,16 @@ bk_status bk_gaussian_loglik(double* a, int64_t n, int64_t ld, const double* z, 
   if (n > (int64_t)65535 * 64)
     return set_error(BK_ERR_INVALID_ARG, "n too large for the tile grid (max %lld)",
                      (long long)65535 * 64);
+  if ((st = check_work(d_work)) != BK_OK) return st;
+  if (d_work != nullptr && work_bytes >= loglik_workspace_bytes(n))
+    return check_cuda(launch_loglik_fixed(a, n, ld, z, y, out, o.d_counters, d_work, s),
+                      "bk_gaussian_loglik");
   return check_cuda(launch_loglik(a, n, ld, z, y, out, o.d_counters, s), "bk_gaussian_loglik");
+}
+
+bk_status bk_gaussian_loglik(double* a, int64_t n, int64_t ld, const double* z, double* y,
+                             double* out, const bk_opts* opts, bk_stream_t stream) {
+  return bk_gaussian_loglik_ws(a, n, ld, z, y, out, opts, nullptr, 0, stream);
 }
 
 bk_status bk_eval(const double* x, const double* nu, double* out, int64_t n, bk_stream_t stream) {

@@ -53,6 +53,12 @@ cudaError_t launch_eval_grad_f64(const double* x, const double* nu, double* k, d
 cudaError_t launch_loglik(double* a, int64_t n, int64_t ld, const double* z, double* y,
                           double* out, unsigned long long* ctr, cudaStream_t s);
 
+// The same with the Cholesky factorisation in fixed point (bk_chol_fixed.cu);
+// work: loglik_workspace_bytes(n), 256-byte aligned.
+size_t loglik_workspace_bytes(int64_t n);
+cudaError_t launch_loglik_fixed(double* a, int64_t n, int64_t ld, const double* z, double* y,
+                                double* out, unsigned long long* ctr, void* work, cudaStream_t s);
+
 // ---- writers with a per-call entry table (bk_entry_table.cu) ----
 // Bytes of a table with FP64 or FP32 records.
 size_t entry_table_bytes(bool f32);
