@@ -29,15 +29,18 @@ __global__ void __launch_bounds__(kTabThreads) entry_table_kernel(
 // i and i + 32 against columns 8 w .. 8 w + 7.  Block (I, J) is stored straight
 // from registers (a warp writes 32 consecutive rows of one column); for a
 // symmetric matrix the tile also goes through shared memory to block (J, I).
-// col_base as in matern_sym_kernel, in tiles of 64.
+// col_base as in matern_sym_kernel, in tiles of 64.  FP32 entries wait on their
+// record's load more than on anything else (n = 40,000: 4 blocks an SM 1,839 us,
+// 5 1,746, 6 1,665, spilling a few registers outside the loop); FP64 entries
+// do not gain from more (n = 20,000: 1,661, 1,654, 1,680).
 template <bool F32, typename OutT, bool kSym>
-__global__ void __launch_bounds__(256, 4) matern_table_kernel(
+__global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
     const unsigned char* __restrict__ table, const double* __restrict__ locs1, int64_t m,
     const double* __restrict__ locs2, int64_t n, const __grid_constant__ MaternParams mp,
     OutT* __restrict__ out, int64_t ld, int64_t tiles_m, int64_t col_base, int width) {
-  __shared__ TabTileSmem<OutT> sm;
+  __shared__ TabTileSmem<F32, OutT> sm;
   const unsigned e0 = tab_first_binade(mp.inv_beta);
-  tab_stage_octaves<F32>(sm.oct, e0);
+  if constexpr (!F32) tab_stage_octaves(sm.pts.oct, e0);
   const unsigned parts = kTabTile / width, tile = blockIdx.x / parts, part = blockIdx.x % parts;
   int64_t I, J;
   if constexpr (kSym) {
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
     const BatchInstance* __restrict__ inst, int count, const int64_t* __restrict__ prefix,
     int64_t limit, unsigned long long* __restrict__ next, int chunk,
     const unsigned char* __restrict__ tables) {
-  __shared__ TabTileSmem<OutT> sm;
+  __shared__ TabTileSmem<F32, OutT> sm;
   __shared__ BatchInstance cur;
   __shared__ int64_t item;
   int k = -1;
@@ -112,7 +115,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
           reinterpret_cast<long long*>(&cur)[threadIdx.x] =
               reinterpret_cast<const long long*>(inst + k)[threadIdx.x];
         __syncthreads();
-        tab_stage_octaves<F32>(sm.oct, tab_first_binade(cur.mp.inv_beta));
+        if constexpr (!F32) tab_stage_octaves(sm.pts.oct, tab_first_binade(cur.mp.inv_beta));
       }
       int64_t I, J;
       tri_tile(w - __ldg(prefix + k), I, J);

@@ -81,6 +81,23 @@ def test_coordinates_of_any_scale(dev, scale, shift, dtype):
     check(got, want)
 
 
+@pytest.mark.parametrize("nu", [0.05, 0.49, 0.5, 3.0])
+@pytest.mark.parametrize("width", [0.5, 7.9, 8.1, 31.0, 63.0, 65.0, 300.0])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_scattered_points(dev, nu, width, dtype):
+    """Unsorted points over 0.5 to 300 beta, so that every tile spans the whole
+    set: on both sides of the spans and distances for which a tile's coordinates
+    are kept relative to it."""
+    g = torch.Generator(device=dev).manual_seed(int(10 * width))
+    L = width * torch.rand((2, 740), generator=g, dtype=torch.float64, device=dev) + 17.0
+    L[:, :200] = L[:, 200:400] + 0.01 * torch.rand((2, 200), generator=g, dtype=torch.float64, device=dev)
+    got = bk.bk_matern_tile(L, 1.0, 1.0, nu, dtype=dtype)
+    want = bk.bk_matern_tile(L, 1.0, 1.0, nu, opts=direct(compute=bk.BK_F64))
+    torch.cuda.synchronize()
+    assert torch.equal(got, got.T)
+    check(got, want)
+
+
 @pytest.mark.parametrize("m,n", [(8192, 64), (63, 9001), (2048, 257), (1, 600000)])
 @pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
 def test_blocks(dev, m, n, dtype):
