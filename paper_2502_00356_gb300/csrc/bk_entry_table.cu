@@ -21,8 +21,9 @@ __global__ void __launch_bounds__(kTabThreads) entry_table_kernel(
     const __grid_constant__ MaternParams mp, const double* __restrict__ locs1, int64_t m,
     const double* __restrict__ locs2, int64_t n, unsigned char* __restrict__ table) {
   __shared__ TabBuildSmem sm;
-  const double r2_max = m + n <= 2 * kTabScan ? tab_r2_bound(sm.box, locs1, m, locs2, n) : kInf;
-  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, r2_max, table);
+  asm volatile("griddepcontrol.launch_dependents;");
+  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, m + n <= 2 * kTabScan, locs1, m, locs2, n,
+                       table);
 }
 
 // One 64 x 64 tile per block of 256 threads; lane i of warp w evaluates rows
@@ -30,17 +31,17 @@ __global__ void __launch_bounds__(kTabThreads) entry_table_kernel(
 // from registers (a warp writes 32 consecutive rows of one column); for a
 // symmetric matrix the tile also goes through shared memory to block (J, I).
 // col_base as in matern_sym_kernel, in tiles of 64.  FP32 entries wait on their
-// record's load more than on anything else (n = 40,000: 4 blocks an SM 1,839 us,
-// 5 1,746, 6 1,665, spilling a few registers outside the loop); FP64 entries
-// do not gain from more (n = 20,000: 1,661, 1,654, 1,680).
+// record's load more than on anything else (n = 40,000: 4 blocks an SM 1,883 us,
+// 6 1,699, 8 1,988, spilling a few registers outside the loop); FP64 entries
+// do not gain from more (n = 20,000: 3 blocks 1,139, 4 1,079, 5 1,081, 6 1,142).
 template <bool F32, typename OutT, bool kSym>
 __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
     const unsigned char* __restrict__ table, const double* __restrict__ locs1, int64_t m,
     const double* __restrict__ locs2, int64_t n, const __grid_constant__ MaternParams mp,
     OutT* __restrict__ out, int64_t ld, int64_t tiles_m, int64_t col_base, int width) {
   __shared__ TabTileSmem<F32, OutT> sm;
-  const unsigned e0 = tab_first_binade(mp.inv_beta);
-  if constexpr (!F32) tab_stage_octaves(sm.pts.oct, e0);
+  // launched while the table's kernel may still run (launch_writer)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const unsigned parts = kTabTile / width, tile = blockIdx.x / parts, part = blockIdx.x % parts;
   int64_t I, J;
   if constexpr (kSym) {
@@ -50,7 +51,7 @@ __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
     I = tile % tiles_m;
     J = tile / tiles_m;
   }
-  tab_tile<F32, OutT, kSym, 8>(sm, table, e0, locs1, m, locs2, n, I, J, mp, out, ld, (int)part, width);
+  tab_tile<F32, OutT, kSym, 8>(sm, table, locs1, m, locs2, n, I, J, mp, out, ld, (int)part, width);
 }
 
 // ---- batched: every instance's constants, tables and tiles in three launches
@@ -82,8 +83,7 @@ __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
   const BatchInstance& b = inst[blockIdx.y];
   if (!b.table) return;
   const MaternParams mp = b.mp;
-  const double r2_max = b.n <= kTabScan ? tab_r2_bound(sm.box, b.locs, b.n, b.locs, b.n) : kInf;
-  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, r2_max,
+  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, b.n <= kTabScan, b.locs, b.n, b.locs, b.n,
                        tables + (size_t)blockIdx.y * TabLayout<F32>::kBytes);
 }
 
@@ -115,13 +115,11 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
           reinterpret_cast<long long*>(&cur)[threadIdx.x] =
               reinterpret_cast<const long long*>(inst + k)[threadIdx.x];
         __syncthreads();
-        if constexpr (!F32) tab_stage_octaves(sm.pts.oct, tab_first_binade(cur.mp.inv_beta));
       }
       int64_t I, J;
       tri_tile(w - __ldg(prefix + k), I, J);
       tab_tile<F32, OutT, true, WARPS>(sm, tables + (size_t)k * TabLayout<F32>::kBytes,
-                                       tab_first_binade(cur.mp.inv_beta), cur.locs, cur.n, cur.locs,
-                                       cur.n, I, J, cur.mp, (OutT*)cur.out, cur.ld, 0, kTabTile,
+                                       cur.locs, cur.n, cur.locs, cur.n, I, J, cur.mp, (OutT*)cur.out, cur.ld, 0, kTabTile,
                                        cur.table != 0);
     }
   }
@@ -131,10 +129,10 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
 
 size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kBytes : TabLayout64::kBytes; }
 
-// entry_table_size (the header): from 2^19 entries on (n = 725) a matrix is worth a table.  The table itself
-// costs about 5 us (its kernel and the launch), what the direct evaluation
-// takes for 2^16 entries; between the two, small matrices keep the direct
-// path, whose results do not depend on whether the caller has scratch memory.
+// entry_table_size (the header): from 2^19 entries on (n = 725) a matrix is worth
+// a table, which costs about 15 us: n = 777 takes 29 us with it, 63 without; at
+// half the entries both take about 25, and such matrices keep the direct path,
+// whose results do not depend on whether the caller has scratch memory.
 bool entry_table_pays(int64_t rows, int64_t cols) { return entry_table_size(rows, cols); }
 
 bool entry_table_applies(const bk_opts& o, double sigma2, double beta, double nu) {
@@ -150,11 +148,27 @@ int tile_width(int64_t ntiles) {
   return ntiles < (int64_t)current_sm_count() * 4 ? kTabTile / 4 : kTabTile;
 }
 
+// Launches a writer so that it may be scheduled while the table's kernel before
+// it still runs (it waits for that kernel's end itself): the launch's latency,
+// about 3 us, is hidden.
+template <typename... P, typename... A>
+cudaError_t launch_writer(void (*kernel)(P...), unsigned grid, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
+
 template <bool F32>
 cudaError_t build_table(const MaternParams& mp, const double* locs1, int64_t m,
                         const double* locs2, int64_t n, unsigned char* table, cudaStream_t s) {
-  constexpr int grid = (TabLayout<F32>::kBins + kTabBinsPerBlock - 1) / kTabBinsPerBlock;
-  entry_table_kernel<F32><<<grid, kTabThreads, 0, s>>>(mp, locs1, m, locs2, n, table);
+  entry_table_kernel<F32><<<current_sm_count(), kTabThreads, 0, s>>>(mp, locs1, m, locs2, n, table);
   return cudaGetLastError();
 }
 
@@ -184,15 +198,13 @@ cudaError_t launch_matern_sym_table(const double* locs, int64_t n, double sigma2
   const int width = tile_width(ntiles);
   const unsigned grid = (unsigned)(ntiles * (kTabTile / width));
   if (f32)
-    matern_table_kernel<true, float, true><<<grid, 256, 0, s>>>(tab, locs, n, locs, n, mp, (float*)out,
-                                                                ld, nb, col_base, width);
-  else if (out_t == BK_F32)
-    matern_table_kernel<false, float, true><<<grid, 256, 0, s>>>(tab, locs, n, locs, n, mp,
-                                                                 (float*)out, ld, nb, col_base, width);
-  else
-    matern_table_kernel<false, double, true><<<grid, 256, 0, s>>>(tab, locs, n, locs, n, mp,
-                                                                  (double*)out, ld, nb, col_base, width);
-  return cudaGetLastError();
+    return launch_writer(matern_table_kernel<true, float, true>, grid, s, tab, locs, n, locs, n, mp,
+                         (float*)out, ld, nb, col_base, width);
+  if (out_t == BK_F32)
+    return launch_writer(matern_table_kernel<false, float, true>, grid, s, tab, locs, n, locs, n, mp,
+                         (float*)out, ld, nb, col_base, width);
+  return launch_writer(matern_table_kernel<false, double, true>, grid, s, tab, locs, n, locs, n, mp,
+                       (double*)out, ld, nb, col_base, width);
 }
 
 cudaError_t launch_matern_block_table(const double* locs1, int64_t m, const double* locs2, int64_t n,
@@ -209,15 +221,13 @@ cudaError_t launch_matern_block_table(const double* locs1, int64_t m, const doub
   const int width = tile_width(tm * tn);
   const unsigned grid = (unsigned)(tm * tn * (kTabTile / width));
   if (f32)
-    matern_table_kernel<true, float, false><<<grid, 256, 0, s>>>(tab, locs1, m, locs2, n, mp,
-                                                                 (float*)out, ld, tm, -1, width);
-  else if (out_t == BK_F32)
-    matern_table_kernel<false, float, false><<<grid, 256, 0, s>>>(tab, locs1, m, locs2, n, mp,
-                                                                  (float*)out, ld, tm, -1, width);
-  else
-    matern_table_kernel<false, double, false><<<grid, 256, 0, s>>>(tab, locs1, m, locs2, n, mp,
-                                                                   (double*)out, ld, tm, -1, width);
-  return cudaGetLastError();
+    return launch_writer(matern_table_kernel<true, float, false>, grid, s, tab, locs1, m, locs2, n, mp,
+                         (float*)out, ld, tm, -1, width);
+  if (out_t == BK_F32)
+    return launch_writer(matern_table_kernel<false, float, false>, grid, s, tab, locs1, m, locs2, n, mp,
+                         (float*)out, ld, tm, -1, width);
+  return launch_writer(matern_table_kernel<false, double, false>, grid, s, tab, locs1, m, locs2, n, mp,
+                       (double*)out, ld, tm, -1, width);
 }
 
 
@@ -228,9 +238,10 @@ namespace {
 template <bool F32, typename OutT>
 cudaError_t launch_batched_table_t(const BatchTable& b, int64_t limit, int warps, int ctas_per_sm,
                                    int chunk, cudaStream_t s) {
-  // 16 (4) blocks share an instance's FP64 (FP32) table: the node weights, once
-  // per block, stay a small part of it
-  batched_table_kernel<F32><<<dim3(F32 ? 4 : 16, (unsigned)b.count), kTabThreads, 0, s>>>(
+  // The instances' tables in one wave of blocks; at least four each, so that the
+  // node weights, once per block, stay a small part of it.
+  const int sms = current_sm_count(), share = b.count < sms / 4 ? sms / b.count : 4;
+  batched_table_kernel<F32><<<dim3((unsigned)share, (unsigned)b.count), kTabThreads, 0, s>>>(
       (const BatchInstance*)b.instances, (unsigned char*)b.tables);
   const int grid = current_sm_count() * ctas_per_sm;
   if (warps == 4)
