@@ -913,6 +913,12 @@ constexpr int kCoshTabSize = 3328;
 static __device__ const double kCoshTab[kCoshTabSize] = {
 #include "bk_cosh_table.inc"
 };
+// h' - h for the same steps, 2 cosh(h') being the rounded entry: the recurrence
+// with that entry runs on nodes j h', and what else is evaluated at j h is off by
+// j (h' - h), which at 30 nodes is most of a sum's error.
+static __device__ const float kCoshShift[kCoshTabSize] = {
+#include "bk_cosh_shift.inc"
+};
 
 // The step h rounded up to 8 significand bits (hq >= h: N hq still covers the
 // window, and the strip bound's error grows by at most e^{2 pi a/h 2^-8},
@@ -1284,7 +1290,7 @@ __device__ __forceinline__ double scale_f64(double xh, double nu, float log2_ove
 // and with the scaled integrand of node_sum_f64,
 //   cosh(t) f/f_s = (D_j / (K x)) f_j / f_s,   t sinh(nu t) e^{-x cosh t} / f_s
 //   = t_j e^{a_j} (1 - e^{-2 nu t_j}),
-// so the node loop carries two more sums (4 more FP64 operations per node).
+// so the node loop carries two more sums.
 // The window must hold the integrand of -dK/dx, which decays like that of
 // K_{nu+1}: it is the union of the windows of orders nu and nu + 1.
 struct NodeSum3 {
@@ -1345,21 +1351,133 @@ __device__ __forceinline__ NodeSum3 node_sum3_f64(double t_start, double H, int 
   return r;
 }
 
-// K, -dK/dx and dK/dnu in scaled form: returns the scale sc and sets
-// hS = h S, hSx = h Sx / (K x) and hSn = h Sn, so that K = e^sc hS,
-// dK/dx = -e^sc hSx, dK/dnu = e^sc hSn.  st / st1: FP32 roots for the orders
-// nu and nu + 1 (both or neither); the window is their union, checked in FP64
-// on K's end nodes as in scale_f64; without roots, or when the check fails,
-// the union of the FP64 search windows.
-__device__ __forceinline__ double scale3_f64(double x, double nu, const double* __restrict__ tab,
-                                             const Start32* st, const Start32* st1,
-                                             double& hS, double& hSx, double& hSn, Tally& tl) {
+// t in [0, 128) in units of 2^-56, truncated.
+__device__ __forceinline__ unsigned long long fix56_f32(float t) {
+  const unsigned b = __float_as_uint(t);
+  const int sh = (int)(b >> 23) - 127 + 33;  // from units of 2^{e-23}
+  const unsigned long long m = (b & 0x7fffffu) | 0x800000u;
+  return sh >= 0 ? m << sh : (sh > -24 ? m >> -sh : 0ULL);
+}
+
+// t (1 - w) for t in units of 2^-56 (below 2^63) and w = Wq 2^-63, on the integer pipe.
+__device__ __forceinline__ double t_minus_w(unsigned long long T, unsigned long long Wq) {
+  const unsigned long long M = __umul64hi(T << 1, (1ULL << 63) - Wq);  // units of 2^-56
+  const int lz = __clzll((long long)M);
+  const unsigned long long q = M << (lz & 63);
+  const long long r = (long long)((q >> 11) + (q >> 10 & 1)) + ((long long)(1023 + 6 - lz) << 52);
+  return M == 0 ? 0.0 : __longlong_as_double(r);
+}
+
+// The three sums without centring, for checked windows: node_sum_cosh (its
+// recurrences, fixed-point parts and conditions; count >= 3, t_j < 128) with two
+// more sums,
+//   Sx = sum_j D_j E_j (1 + W_j)  (K x cosh t_j),  Sn = sum_j t_j E_j (1 - W_j),
+// t_j (1 - W_j) from the integer pipe as W_j is.  A node costs 5 FP64 operations
+// (the D recurrence, D (1 + W), three sums) where node_sum3_f64 takes 12: that
+// loop kept the FP64 pipe 85 % busy.
+struct NodeSum3C {
+  double S, Sx, Sn;         // end weights 1/2 included
+  float l2_first, l2_last;  // as NodeSumC
+  bool pos;
+};
+__device__ __forceinline__ NodeSum3C node_sum3_cosh(float t0f, float hq, int count, double xh, double nu,
+                                                    const double* __restrict__ tab, int step_idx) {
+  const double t_start = widen_f(t0f), H = widen_f(hq);
+  const bool start_pos = t0f > 0.0f;
+  double c, D0, D1, W = 1.0;
+  unsigned long long Wq = 1ULL << 63;
+  if (start_pos) {
+    const double e0 = exp_acc(t_start, tab), r0 = rcp_nr2(e0);
+    const double eh = exp_acc(H, tab), rh = rcp_nr2(eh);
+    c = step_idx >= 0 ? kCoshTab[step_idx] : bits_le(H, 0.35) ? two_cosh_small(H) : eh + rh;
+    D0 = xh * (e0 + r0);
+    D1 = xh * fma(e0, eh, r0 * rh);
+    W = exp_acc(fmax(-2.0 * nu * t_start, -708.0), tab);
+    Wq = fix63_unit(W);
+  } else {
+    c = (step_idx >= 0) ? kCoshTab[step_idx] : two_cosh_warp(H, tab);
+    D0 = __hiloint2double(__double2hiint(xh) + (1 << 20), __double2loint(xh));
+    D1 = xh * c;
+  }
+  const unsigned long long Rq = fix64_unit(decay_step(nu, H, tab));
+  // nu t_j on the nodes of the recurrence with c (rms errors 8e-14 -> 3e-14)
+  const double Hs = step_idx >= 0 ? H + widen_f(kCoshShift[step_idx]) : H;
+  const long long Gs = __double2ll_rn(nu * Hs * kExpScale40);
+  const unsigned long long Ts = fix56_f32(hq);
+  unsigned long long T = fix56_f32(t0f);
+  long long G = 0;
+  NodeSum3C r;
+  double s = exp2s_fix<0>(fix40_node(D0), tab), sn = 0.0;
+  r.l2_first = 0.0f;
+  if (start_pos) {
+    const double C0h = fma(W, 0.5, 0.5);
+    r.l2_first = log2_f64_approx(s) + log2_f64_approx(C0h) + 1.0f;
+    sn = s * (t_start * fma(W, -0.5, 0.5));
+    s *= C0h;
+  }
+  double sx = D0 * s;
+#pragma unroll 1  // (two nodes in flight cost registers: 409 us against 401 for 10^6 pairs)
+  for (int j = 1; j < count - 1; ++j) {
+    const double D2 = fma(c, D1, -D0);
+    D0 = D1;
+    D1 = D2;
+    G += Gs;
+    T += Ts;
+    Wq = __umul64hi(Wq, Rq);
+    const double E = exp2s_fix<0>(fix40_node(D0) - G, tab), w = one_plus_w(Wq);
+    s = fma(E, w, s);
+    sx = fma(E, D0 * w, sx);
+    sn = fma(E, t_minus_w(T, Wq), sn);
+  }
+  {
+    G += Gs;
+    T += Ts;
+    Wq = __umul64hi(Wq, Rq);
+    const double Eh = exp2s_fix<-1>(fix40_node(D1) - G, tab), w = one_plus_w(Wq);
+    s = fma(Eh, w, s);
+    sx = fma(Eh, D1 * w, sx);
+    sn = fma(Eh, t_minus_w(T, Wq), sn);
+    r.l2_last = log2_f64_approx(Eh) + log2_f64_approx(w) + 1.0f;
+    r.pos = bits_pos(Eh);
+  }
+  r.S = s;
+  r.Sx = sx;
+  r.Sn = sn;
+  return r;
+}
+
+// Whether computed end terms (log2, unweighted; of a node sum whose scale is
+// e^{nu t0}) meet the window's rule: see scale_f64.
+__device__ __forceinline__ bool ends_ok(float xf, float nuf, const Start32& st, float t0f, float tnf,
+                                        float l2_first, float l2_last) {
+  constexpr float kL2e = 1.44269504f;
+  const float G = fmaf(nuf, st.ts - t0f, -xf * st.cs) * kL2e;  // log2 of the peak term
+  float w1, lw1;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w1) : "f"(-2.0f * kL2e * nuf * tnf));
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lw1) : "f"(1.0f + w1));
+  if (!(l2_last - lw1 - G <= -52.0f)) return false;
+  if (!(t0f > 0.0f)) return true;
+  float w0, lw0;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(w0) : "f"(-2.0f * kL2e * nuf * t0f));
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lw0) : "f"(1.0f + w0));
+  return l2_first - lw0 - G <= -53.0f;
+}
+
+// K, -dK/dx and dK/dnu in scaled form, centred at t*: the rare path of
+// scale3_f64.  check: the window is the union of the FP32 roots' for the orders nu
+// and nu + 1, checked in FP64 on K's end nodes as in scale_f64; without, or when
+// the check fails, the union of the FP64 search windows.
+struct Scaled3 {
+  double scale, hS, hSx, hSn;
+};
+static __device__ __noinline__ Scaled3 scale3_centred(double x, double nu, const double* __restrict__ tab,
+                                                      bool check, Start32 st, Start32 st1, Tally& tl) {
+  Scaled3 r;
   constexpr double kEps64 = 0x1p-52;
   Window64 w;
-  bool check = (st != nullptr && st1 != nullptr);
   if (check) {
-    w = window_from_start(x, nu, *st, tab);
-    const Window64 w1 = window_from_start(x, nu + 1.0, *st1, tab);
+    w = window_from_start(x, nu, st, tab);
+    const Window64 w1 = window_from_start(x, nu + 1.0, st1, tab);
     w.t0 = fmin(w.t0, w1.t0);
     w.t1 = fmax(w.t1, w1.t1);
   }
@@ -1380,8 +1498,8 @@ __device__ __forceinline__ double scale3_f64(double x, double nu, const double* 
         continue;
       }
       ++tl.fail;
-      hS = hSx = hSn = __longlong_as_double(0x7ff8000000000000LL);
-      return hS;
+      r.scale = r.hS = r.hSx = r.hSn = __longlong_as_double(0x7ff8000000000000LL);
+      return r;
     }
     const double h = width * rcp_nr2((double)N);
     const NodeSum3 ns = node_sum3_f64(w.t0, h, N + 1, x, nu, w.ts, w.cs, tab);
@@ -1392,12 +1510,60 @@ __device__ __forceinline__ double scale3_f64(double x, double nu, const double* 
       check = false;
       continue;
     }
-    hS = h * (ns.S - 0.5 * (ns.f0 + ns.fN));
-    hSx = h * (ns.Sx - 0.5 * (ns.fx0 + ns.fxN)) * rcp_nr2(kExpScale * x);
-    hSn = h * (ns.Sn - 0.5 * (ns.fn0 + ns.fnN));
+    r.hS = h * (ns.S - 0.5 * (ns.f0 + ns.fN));
+    r.hSx = h * (ns.Sx - 0.5 * (ns.fx0 + ns.fxN)) * rcp_nr2(kExpScale * x);
+    r.hSn = h * (ns.Sn - 0.5 * (ns.fn0 + ns.fnN));
     break;
   }
-  return fma(nu, w.ts, -x * w.cs) - kLn2;
+  r.scale = fma(nu, w.ts, -x * w.cs) - kLn2;
+  return r;
+}
+
+// K, -dK/dx and dK/dnu in scaled form: returns the scale sc and sets
+// hS = h S, hSx = h Sx / (K x) and hSn = h Sn, so that K = e^sc hS,
+// dK/dx = -e^sc hSx, dK/dnu = e^sc hSn.  st / st1: FP32 roots for the orders
+// nu and nu + 1 (both or neither); the window is their union with scale_f64's
+// geometry and check, the sums node_sum3_cosh's where cosh_loop_ok; scale3_centred
+// elsewhere.  100,000 pairs: 125 -> 64 us, 10^6: 949 -> 401.
+__device__ __forceinline__ double scale3_f64(double x, double nu, const double* __restrict__ tab,
+                                             const Start32* st, const Start32* st1,
+                                             double& hS, double& hSx, double& hSn, Tally& tl) {
+  const bool starts = st != nullptr && st1 != nullptr;
+  if (starts) {
+    auto left = [](const Start32& a) {
+      return (a.t0 > 0.0f && a.ts > 0.0f) ? fmaxf(0.0f, fmaf(a.t0, -2e-5f, a.t0) - 1e-5f) : 0.0f;
+    };
+    const float t1 = fmaxf(st->t1, st1->t1), t1f = fmaf(t1, 2e-5f, t1) + 1e-5f;
+    const float t0f = fminf(left(*st), left(*st1)), wf = t1f - t0f;
+    const float xf = f32_trunc(x), nuf = f32_trunc(nu);
+    // (the rounded-up step costs up to a factor 1.13 of the strip bound; half a unit
+    // of its exponent, 2 % more nodes, makes up for it and for the coarser exponent)
+    const int N = strip_node_count(xf, nuf + 1.0f, wf, kPlainLog2OverTol + 0.5f, kPlainMaxNodes);
+    if (N <= kPlainMaxNodes) {
+      int step_idx;
+      const float hq = quantise_step(__fdividef(wf, (float)N), step_idx);
+      const float tnf = fmaf((float)N, hq, t0f);
+      if (cosh_loop_ok(xf, nuf, t0f, tnf, N) && tnf < 127.0f) {
+        const double xh = (0.5 * kExpScale) * x;
+        const NodeSum3C ns = node_sum3_cosh(t0f, hq, N + 1, xh, nu, tab, step_idx);
+        tl.nodes += N + 1;
+        if (ns.pos && ends_ok(xf, nuf, *st, t0f, tnf, ns.l2_first, ns.l2_last) && bits_pos(ns.S) &&
+            bits_le(ns.S, 1e300)) {
+          const double h = widen_f(0.5f * hq);
+          hS = h * ns.S;
+          hSx = (h * ns.Sx) * rcp_nr2(kExpScale * x);
+          hSn = bits_pos(nu) ? h * ns.Sn : 0.0;
+          return t0f > 0.0f ? nu * widen_f(t0f) : 0.0;
+        }
+        ++tl.fallback;
+      }
+    }
+  }
+  const Scaled3 r = scale3_centred(x, nu, tab, starts, starts ? *st : Start32{}, starts ? *st1 : Start32{}, tl);
+  hS = r.hS;
+  hSx = r.hSx;
+  hSn = r.hSn;
+  return r.scale;
 }
 
 // The paper's fixed window (Algorithm 2, x >= 0.1 branch, Sec. IV-C): the
