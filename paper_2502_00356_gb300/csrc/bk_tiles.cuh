@@ -7,6 +7,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "bk.h"
@@ -75,6 +76,12 @@ __device__ __forceinline__ Form bind_table(const Form& form, double* s_tab) {
   return f;
 }
 
+// The block's size: kBlock, or where that is 0 the launch's.
+template <int kBlock>
+__device__ __forceinline__ int block_size() {
+  return kBlock > 0 ? kBlock : (int)blockDim.x;
+}
+
 constexpr int kSortChunk = 1024;  // pairs per counting sort (8 rounds of 128)
 
 // Orders the pairs [lo, lo + cnt), cnt <= kSortChunk, by bucket_of(x, nu) in
@@ -83,15 +90,15 @@ constexpr int kSortChunk = 1024;  // pairs per counting sort (8 rounds of 128)
 // order inside a bucket).  Warps that then take consecutive runs of 32 see
 // similar node counts and search paths, where random pairs leave most lanes
 // idle while the slowest finishes.  Each pair's arithmetic is unchanged and
-// results go back to their own positions.  Every thread of the 128-thread
-// block calls it; x and nu are read again from L1 in the rounds that follow.
-template <class BucketOf>
+// results go back to their own positions.  Every thread of the block (128 or
+// more) calls it; x and nu are read again from L1 in the rounds that follow.
+template <int kBlock, class BucketOf>
 __device__ __forceinline__ void sort_chunk(const double* __restrict__ x,
                                            const double* __restrict__ nu, int64_t lo, int cnt,
                                            unsigned short* s_perm, unsigned* s_cnt,
                                            BucketOf bucket_of) {
   constexpr int kR = kSortChunk / 128;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, nt = block_size<kBlock>();
   __syncthreads();  // the previous chunk's order is no longer read
   if (t < 64) s_cnt[t] = 0u;
   __syncthreads();
@@ -99,7 +106,7 @@ __device__ __forceinline__ void sort_chunk(const double* __restrict__ x,
   unsigned char bk[kR];
 #pragma unroll
   for (int r = 0; r < kR; ++r) {
-    const int k = r * 128 + t;
+    const int k = r * nt + t;
     bk[r] = 0;
     rank[r] = 0;
     if (k < cnt) {
@@ -123,38 +130,40 @@ __device__ __forceinline__ void sort_chunk(const double* __restrict__ x,
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < kR; ++r) {
-    const int k = r * 128 + t;
+    const int k = r * nt + t;
     if (k < cnt) s_perm[s_cnt[bk[r]] + rank[r]] = (unsigned short)k;
   }
   __syncthreads();
 }
 
-// The sorted position thread t takes in round r of a sorted chunk: warp w
-// takes run 4r + w in even rounds and run 4r + 3 - w in odd ones, so that
-// the four warps get equal shares of cheap and costly runs.
+// The sorted position thread t takes in round r of a sorted chunk: with W warps,
+// warp w takes run W r + w in even rounds and run W r + W - 1 - w in odd ones, so
+// that the warps get equal shares of cheap and costly runs.
+template <int kBlock>
 __device__ __forceinline__ int sorted_slot(int r) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  return (4 * r + ((r & 1) ? 3 - w : w)) * 32 + l;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = block_size<kBlock>() >> 5;
+  return (nw * r + ((r & 1) ? nw - 1 - w : w)) * 32 + l;
 }
 
 // Block b's pairs [lo, hi) when the grid (one wave of resident blocks) takes
-// the n pairs in equal contiguous chunks of whole 128-pair rounds (+9 % on
-// 10^7 FP64 evaluations over a grid-stride loop).
+// the n pairs in equal contiguous chunks of whole rounds (+9 % on 10^7 FP64
+// evaluations over a grid-stride loop).
+template <int kBlock>
 __device__ __forceinline__ void block_range(int64_t n, int64_t& lo, int64_t& hi) {
-  const int64_t chunk = ((n + gridDim.x - 1) / gridDim.x + 127) / 128 * 128;
+  const int64_t nt = block_size<kBlock>(), chunk = ((n + gridDim.x - 1) / gridDim.x + nt - 1) / nt * nt;
   lo = (int64_t)blockIdx.x * chunk;
   hi = lo + chunk < n ? lo + chunk : n;
 }
 
-// Bare evaluations of the FP64 forms, 128 per block and round, in chunks
+// Bare evaluations of the FP64 forms, one per thread and round, in chunks
 // sorted by the form's cost bucket (sort_chunk).
-template <class Form, typename OutT>
-__global__ void __launch_bounds__(128, 6) eval_kernel(const Form form, const double* __restrict__ x,
+template <class Form, typename OutT, int kBlock>
+__global__ void __launch_bounds__(kBlock == 128 ? 128 : 256, kBlock == 128 ? 6 : 3) eval_kernel(const Form form, const double* __restrict__ x,
                                                    const double* __restrict__ nu,
                                                    OutT* __restrict__ out,
                                                    OutT* __restrict__ log_out, int64_t n,
                                                    unsigned long long* __restrict__ ctr) {
-  constexpr int kB = 128;
+  const int kB = block_size<kBlock>();
   __shared__ double s_tab[Form::kStageTable ? kExpTabSize : 1];
   __shared__ unsigned short s_perm[kSortChunk];
   __shared__ unsigned s_cnt[64];
@@ -163,14 +172,14 @@ __global__ void __launch_bounds__(128, 6) eval_kernel(const Form form, const dou
   unsigned evals = 0;
   const bool want_log = (log_out != nullptr);
   int64_t lo, hi;
-  block_range(n, lo, hi);
+  block_range<kBlock>(n, lo, hi);
   for (int64_t base = lo; base < hi; base += kSortChunk) {
     const int cnt = (int)(hi - base < kSortChunk ? hi - base : kSortChunk);
-    sort_chunk(x, nu, base, cnt, s_perm, s_cnt,
+    sort_chunk<kBlock>(x, nu, base, cnt, s_perm, s_cnt,
                [&](double xi, double vi) { return f.sort_bucket(xi, vi); });
     const int rounds = (cnt + kB - 1) / kB;
     for (int r = 0; r < rounds; ++r) {
-      const int p = sorted_slot(r);
+      const int p = sorted_slot<kBlock>(r);
       if (p < cnt) {
         const int64_t i = base + s_perm[p];
         OutT k, lk;
@@ -218,18 +227,18 @@ __global__ void __launch_bounds__(128, 8) eval_coop_kernel(const Form form,
   flush_tally(ctr, tl, evals);
 }
 
-// K, dK/dx and dK/dnu of the plain form, 128 pairs per block and round, in
+// K, dK/dx and dK/dnu of the plain form, one pair per thread and round, in
 // chunks sorted by the cost bucket (sort_chunk).  Domain: x = 0 gives (+inf,
 // -inf, NaN), x = +inf gives (0, 0, 0), x < 0 or NaN and non-finite nu give
 // NaN; dK/dnu is odd in nu (K_{-nu} = K_nu).  Null outputs are skipped.
 template <class Form>
-__global__ void __launch_bounds__(128, 4) eval_grad_kernel(const Form form, const double* __restrict__ x,
+__global__ void __launch_bounds__(256, 2) eval_grad_kernel(const Form form, const double* __restrict__ x,
                                                         const double* __restrict__ nu,
                                                         double* __restrict__ k,
                                                         double* __restrict__ dkdx,
                                                         double* __restrict__ dkdnu, int64_t n,
                                                         unsigned long long* __restrict__ ctr) {
-  constexpr int kB = 128;
+  const int kB = block_size<0>();
   __shared__ double s_tab[Form::kStageTable ? kExpTabSize : 1];
   __shared__ unsigned short s_perm[kSortChunk];
   __shared__ unsigned s_cnt[64];
@@ -238,14 +247,14 @@ __global__ void __launch_bounds__(128, 4) eval_grad_kernel(const Form form, cons
   unsigned evals = 0;
   const double qnan = __longlong_as_double(0x7ff8000000000000LL);
   int64_t lo, hi;
-  block_range(n, lo, hi);
+  block_range<0>(n, lo, hi);
   for (int64_t base = lo; base < hi; base += kSortChunk) {
     const int cnt = (int)(hi - base < kSortChunk ? hi - base : kSortChunk);
-    sort_chunk(x, nu, base, cnt, s_perm, s_cnt,
+    sort_chunk<0>(x, nu, base, cnt, s_perm, s_cnt,
                [](double xi, double vi) { return eval_cost_bucket(xi, vi); });
     const int rounds = (cnt + kB - 1) / kB;
     for (int r = 0; r < rounds; ++r) {
-      const int p = sorted_slot(r);
+      const int p = sorted_slot<0>(r);
       if (p >= cnt) continue;
       const int64_t i = base + s_perm[p];
       const double xi = x[i], vi = nu[i], av = fabs(vi);
@@ -466,13 +475,25 @@ inline int tile_grid(int64_t ntiles, int per_block) {
 // Blocks for a grid-stride launch: min(work, SMs x per_sm).
 int grid_for(int64_t work_items, int per_sm);
 
-// The grid of one wave of per_sm blocks per SM for n pairs in rounds of 128,
-// with no block left without a round (block_range).
-inline int one_wave_grid(int64_t n, int per_sm) {
-  const int64_t slots = (int64_t)current_sm_count() * per_sm;
-  const int64_t rounds = (n + 127) / 128;
-  const int64_t per = (rounds + slots - 1) / slots;  // rounds per block
-  return (int)((rounds + per - 1) / per);
+// Grid and block of the sorted kernels, in one wave: blocks of 128 threads, per_sm
+// of them on an SM at once, each with an equal number of rounds and none without
+// (block_range); or, where that gives every SM fewer runs of 32 pairs, the fewest
+// blocks of up to eight warps that hold all pairs at once: 100,000 pairs are 21
+// runs an SM in three blocks of seven warps, where blocks of 128 put 24 on some
+// SMs (38.5 -> 34.6 us).  Blocks of fewer than four warps would sort too few pairs
+// (1,000 evaluations in blocks of 64 took 27.4 us, in blocks of 128 25.5).
+struct WaveShape {
+  int grid, block;
+};
+inline WaveShape one_wave_shape(int64_t n, int per_sm) {
+  auto up = [](int64_t a, int64_t b) { return (a + b - 1) / b; };
+  const int64_t sms = current_sm_count(), warps = up(n, 32 * sms);  // an SM's
+  const int64_t rounds = up(n, 128), per = up(rounds, sms * per_sm), grid = up(rounds, per);
+  if (warps <= 4 * per_sm) {
+    const int64_t blocks = up(warps, 8), block = 32 * std::max<int64_t>(up(warps, blocks), 4);
+    if (blocks * block < up(grid, sms) * per * 128) return WaveShape{(int)up(n, block), (int)block};
+  }
+  return WaveShape{(int)grid, 128};
 }
 
 template <class Form, typename OutT>
@@ -503,13 +524,16 @@ cudaError_t launch_eval_form(const Form& form, const double* x, const double* nu
   } else {
     // one wave of the resident slots (6 blocks per SM), each block taking an
     // equal contiguous chunk of whole rounds (block_range)
-    const int grid = one_wave_grid(n, 6);
+    const WaveShape w = one_wave_shape(n, 6);
+    auto launch = [&](auto kernel, auto* o, auto* lo) {
+      kernel<<<w.grid, w.block, 0, s>>>(form, x, nu, o, lo, n, ctr);
+    };
     if (out_t == BK_F64)
-      eval_kernel<Form, double><<<grid, 128, 0, s>>>(form, x, nu, (double*)out, (double*)log_out,
-                                                     n, ctr);
+      launch(w.block == 128 ? eval_kernel<Form, double, 128> : eval_kernel<Form, double, 0>, (double*)out,
+             (double*)log_out);
     else
-      eval_kernel<Form, float><<<grid, 128, 0, s>>>(form, x, nu, (float*)out, (float*)log_out, n,
-                                                    ctr);
+      launch(w.block == 128 ? eval_kernel<Form, float, 128> : eval_kernel<Form, float, 0>, (float*)out,
+             (float*)log_out);
     return cudaGetLastError();
   }
 }
