@@ -80,6 +80,13 @@ CholLayout chol_layout(int64_t n) {
   return l;
 }
 
+// Each kernel of the chain is launched while the one before it still runs, waits
+// here for that one's end (and so for all before it), and then lets the next one
+// come: the launches' latency, about 2 us each, is hidden.
+__device__ __forceinline__ void chain() {
+  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ double qnan() { return __longlong_as_double(0x7ff8000000000000LL); }
 
 // a 2^{60 - s_i - s_j} as an integer (rounded); false when it is not below 2^60.
@@ -320,6 +327,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
   PanelSmem& sm = *reinterpret_cast<PanelSmem*>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t o = k * kNB;
+  chain();
   if ((int)blockIdx.x == row_blocks) {
     finish_panel(a, ld, n, k - 1, y, w, reinterpret_cast<double*>(smem_raw));
     return;
@@ -628,6 +636,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
   __syncthreads();
   tc::fence_after();
   const uint32_t tm = bar.tmem;
+  chain();
   const int nt = (int)((n + kNB - 1) / kNB), ki = (int)k, workers = (int)gridDim.x;
   const int t0 = (int)(tiles * blockIdx.x / workers), t1 = (int)(tiles * (blockIdx.x + 1) / workers);
   int I = (ki + 1) / 2, left = t0;  // the first tile's row block and place in it
@@ -785,6 +794,7 @@ __global__ void __launch_bounds__(kPanelThreads) chol_finish_kernel(
     double* __restrict__ a, int64_t ld, int64_t n, int64_t nt, double* __restrict__ y,
     double* __restrict__ out, CholWork w, unsigned long long* __restrict__ ctr) {
   __shared__ double sh[kNB * (kNB + 1) + 8 * kNB];
+  chain();
   finish_panel(a, ld, n, nt - 1, y, w, sh);
   if (threadIdx.x >= 32) return;
   __syncwarp();
@@ -807,6 +817,22 @@ __global__ void __launch_bounds__(kPanelThreads) chol_finish_kernel(
   out[1] = 2.0 * ld_;
   out[2] = q;
   out[0] = -0.5 * (q + 2.0 * ld_ + (double)n * 1.8378770664093454836);  // log 2 pi
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), int64_t grid, int block, size_t smem, cudaStream_t s,
+                           A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
 }
 
 // Shared memory beyond 48 KB: opted in once per device.
@@ -851,16 +877,17 @@ cudaError_t launch_loglik_fixed(double* a, int64_t n, int64_t ld, const double* 
     const int extra = k == 0 ? 0 : k == 1 ? 1 : 1 + (int)((n - k * kNB + 255) / 256);
     const auto panel = k == 0 ? (wide ? chol_panel_kernel<true, 5> : chol_panel_kernel<true, 4>)
                               : (wide ? chol_panel_kernel<false, 5> : chol_panel_kernel<false, 4>);
-    panel<<<(unsigned)(row_blocks + extra), kPanelThreads, sizeof(PanelSmem), s>>>(a, ld, n, k, row_blocks,
-                                                                                   rows, y, w);
+    e = launch_chained(panel, row_blocks + extra, kPanelThreads, sizeof(PanelSmem), s, a, ld, n, k,
+                       row_blocks, rows, y, w);
+    if (e != cudaSuccess) return e;
     if (below <= 0) break;
     int64_t tiles = 0;
     for (int I = (int)(k + 1) / 2; I < R; ++I) tiles += row_tiles(I, (int)k, (int)nt);
     const auto update = k == 0 ? chol_update_kernel<true> : chol_update_kernel<false>;
-    update<<<(unsigned)(tiles < sms ? tiles : sms), kUpdThreads, kUpdSmem, s>>>(a, ld, n, k, tiles, w);
+    e = launch_chained(update, tiles < sms ? tiles : sms, kUpdThreads, kUpdSmem, s, a, ld, n, k, tiles, w);
+    if (e != cudaSuccess) return e;
   }
-  chol_finish_kernel<<<1, kPanelThreads, 0, s>>>(a, ld, n, nt, y, out, w, ctr);
-  return cudaGetLastError();
+  return launch_chained(chol_finish_kernel, 1, kPanelThreads, 0, s, a, ld, n, nt, y, out, w, ctr);
 }
 
 }  // namespace bk
