@@ -33,6 +33,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "bk_internal.h"
@@ -53,7 +54,7 @@ constexpr int kRowBlock = 128;   // rows of an MMA tile and of a slice block
 constexpr int kSliceBytes = kRowBlock * kNB * 2;           // 16,384
 constexpr int kBlockBytes = kSlices * kSliceBytes;         // 114,688
 constexpr int kPanelThreads = 512;
-constexpr int kEpiWarps = 8;
+constexpr int kEpiWarps = 16;
 constexpr int kEpiCols = kNB / (kEpiWarps / 4);            // columns of an epilogue thread
 constexpr int kUpdThreads = (kEpiWarps + 2) * 32;          // epilogue, MMA, copies
 constexpr long long kWaitCycles = 2000000000LL;            // bound of every barrier wait, about 1 s
@@ -279,7 +280,8 @@ __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld,
 
 // ---------------------------------------------------------------------------
 // A panel.  Block b < row_blocks factors the diagonal tile (rows 0 .. 63 of its
-// shared array) and solves rows_per_block rows below it (rows 64 ..) against it, in
+// shared array) and solves rows_per_block rows below it (rows 64 .., none for the
+// last block, which writes the tile instead) against it, in
 // column groups of 8.  The pivots are one serial chain (about 400 cycles a
 // column: root, scaling, update of the next pivot), so everything else is
 // arranged around it.  Four (kSolve) solving warps, one on each of the SM's
@@ -353,25 +355,34 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
   const int64_t r0 = o + kNB + (int64_t)blockIdx.x * rows_per_block;
   int own = 0;
   if (r0 < n) own = (int)(n - r0 < rows_per_block ? n - r0 : rows_per_block);
-  if (tid == 0) sm.bad = *w.flag != 0;
-  if (tid < kNB) {
-    sm.scale[tid] = tid < b ? w.scale[o + tid] : 0;
-    sm.scale[kNB + tid] = tid < own ? w.scale[r0 + tid] : 0;
-  }
-  __syncthreads();
   {
-    const int row = tid & 127;
+    // All 16 loads of a thread go out before the first is waited for: four at a
+    // time, behind the scales, they took 3 us (now 1.8).
+    const int row = tid & 127, q = tid >> 7;
     const bool diag = row < kNB;
     const int64_t r = diag ? o + row : r0 + row - kNB;
     const bool in = diag ? row < b : row - kNB < own;
+    constexpr int kEach = kNB / (kPanelThreads / 128);
+    double x[kEach];
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+      const int c = q + i * (kPanelThreads / 128);
+      x[i] = in && c < b && (!diag || c <= row) ? a[r + (o + c) * ld] : 0.0;
+    }
+    if (tid == 0) sm.bad = *w.flag != 0;
+    if (tid < 2 * kNB) sm.scale[tid] = in ? w.scale[r] : 0;
+    if constexpr (kFirst) __syncthreads();
     bool ok = true;
-#pragma unroll 4
-    for (int c = tid >> 7; c < kNB; c += kPanelThreads / 128) {
-      long long v = 0;
-      if (in && c < b && (!diag || c <= row)) {
-        const double x = a[r + (o + c) * ld];
-        if constexpr (kFirst) ok = to_fixed(x, sm.scale[row] + sm.scale[c], v) && ok;
-        else v = __double_as_longlong(x);
+#pragma unroll
+    for (int i = 0; i < kEach; ++i) {
+      const int c = q + i * (kPanelThreads / 128);
+      long long v;
+      if constexpr (kFirst) {
+        v = 0;
+        if (in && c < b && (!diag || c <= row))
+          ok = to_fixed(x[i], sm.scale[row] + sm.scale[c], v) && ok;
+      } else {
+        v = __double_as_longlong(x[i]);
       }
       if (diag && c == row && row >= b) v = 1LL << 58;  // identity beyond the matrix
       sm.S[row][c] = v;
@@ -463,7 +474,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
     __syncthreads();
   }
   const bool bad = sm.bad != 0;
-  if (blockIdx.x == 0) {
+  if ((int)blockIdx.x == row_blocks - 1) {
     if (bad && tid == 0) *w.flag = 1;
     for (int e = tid; e < kNB * kNB; e += kPanelThreads) {
       const int r = e & 63, c = e >> 6;
@@ -510,15 +521,17 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
 // The trailing update N_ij -= x_i x_j^T over the panel's 64 columns, in tiles of
 // 128 rows x 64 columns: the rows' seven slices (112 KB) stay in shared memory
 // along a row of tiles, the columns' (56 KB) are double-buffered, both by bulk
-// copies from one warp.  One thread issues the 34 digit products (K = 64, four
-// MMAs each) into eight accumulators of 64 TMEM columns, S_7 first; eight warps
-// drain each accumulator as it completes into 64-bit integers, so that the next
-// tile's products overlap this tile's epilogue.  An MMA takes 68 cycles of operand
-// fetch, a tile 9,200, which bounds n = 8,000; a tile alone is 15 us (fill, one
-// drain), which with the panel's 28 us bounds n = 1,000.  Sixteen warps drained
-// no faster.
+// copies from one warp.  The 34 digit products (K = 64) go into eight accumulators of
+// 64 TMEM columns, S_0 .. S_7 side by side, so that slice s of the rows times slices
+// t .. t + c - 1 of the columns is one MMA of N = 64 c into S_{s+t} and the next: 48 of
+// them, 4,352 cycles.  As 136 MMAs of N = 64 they took 60 to 68 cycles each, rows in
+// shared memory or in TMEM, against 32 of arithmetic.  S_g is complete after slice
+// g, and sixteen warps drain it into 64-bit integers while the products go on, the
+// next tile's too.  The drain (about 700 cycles a sum) and the entries' loads and
+// stores bound it: a tile among many takes 4.3 us (5.9 with 136 MMAs, a conversion
+// of every sum and eight warps), at n = 8,000 two thirds of HBM's rate for the entries.
 struct UpdBarriers {
-  uint64_t full_a, full_b[2], free_b[2], done[kGroups], drained[kGroups], last;
+  uint64_t full_a[kSlices], full_b[2], free_b[2], done[kGroups], drained[kGroups], last;
   uint32_t tmem;
 };
 constexpr int kBBytes = kBlockBytes / 2;
@@ -597,6 +610,14 @@ __device__ __forceinline__ void store_if(double* p, long long v, int c, int cols
                : "memory");
 }
 
+// Sums of magnitude below 2^22 become integers by adding 1.5 2^23, whose bits they
+// then follow (a conversion has an eighth of the addition's rate); what those bits
+// add to an entry, S_1's in the upper word and S_6's and S_7's below, goes off at once.
+constexpr float kMagic = 12582912.0f;
+constexpr unsigned kMagicBits = 0x4B400000u;
+constexpr unsigned long long kMagicSum =
+    ((unsigned long long)(kMagicBits << 7) << 32) + 2ULL * kMagicBits;
+
 // One lane of the (converged) warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
@@ -620,7 +641,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
   UpdBarriers& bar = *reinterpret_cast<UpdBarriers*>(smem + kBlockBytes + 2 * kBBytes);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
-    tc::mbar_init(&bar.full_a, 1);
+    for (int s = 0; s < kSlices; ++s) tc::mbar_init(&bar.full_a[s], 1);
     tc::mbar_init(&bar.full_b[0], 1);
     tc::mbar_init(&bar.full_b[1], 1);
     tc::mbar_init(&bar.free_b[0], 1);
@@ -650,69 +671,86 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
   };
   if (warp == kEpiWarps + 1) {
     if (lane == 0) {  // the copies: tile t's into buffer t mod 2 once tile t - 2's products are complete
-      int cur = -1;
+      int cur = -1, loads = 0, it = 0;
       bool ok = true;
-      for (int t = t0; t < t1 && ok; ++t) {
-        const int it = t - t0, buf = it & 1;
-        // tile t - 2's products are complete (always waited for: a parity is only
-        // unambiguous one phase ahead) ...
+      for (; it < t1 - t0; ++it) {
+        const int buf = it & 1;
         if (it > 1) ok = wait_phase(&bar.free_b[buf], (uint32_t)((it >> 1) - 1) & 1u);
-        // ... and tile t - 1's before the rows' digits are replaced
-        if (ok && it > 0 && I != cur) ok = wait_phase(&bar.done[0], (uint32_t)(it - 1) & 1u);
         if (!ok) break;
-        if (I != cur) {
-          expect_tx(&bar.full_a, kBlockBytes);
-          bulk_copy(A, w.slices + (size_t)I * kBlockBytes, kBlockBytes, &bar.full_a);
-          cur = I;
-        }
         // the column block is half of a 128-row block in each slice
         const unsigned char* src = w.slices + (size_t)(J / 2) * kBlockBytes + (J & 1) * (kSliceBytes / 2);
         expect_tx(&bar.full_b[buf], kBBytes);
         for (int s = 0; s < kSlices; ++s)
           bulk_copy(B + buf * kBBytes + s * (kSliceBytes / 2), src + s * kSliceBytes, kSliceBytes / 2,
                     &bar.full_b[buf]);
+        if (I != cur) {  // each of the rows' slices once tile t - 1 is through with it
+          src = w.slices + (size_t)I * kBlockBytes;
+          for (int s = 0; s < kSlices; ++s) {
+            if (it > 0) ok = ok && wait_phase(&bar.done[s], (uint32_t)(it - 1) & 1u);
+            if (!ok) break;
+            expect_tx(&bar.full_a[s], kSliceBytes);
+            bulk_copy(A + s * kSliceBytes, src + s * kSliceBytes, kSliceBytes, &bar.full_a[s]);
+          }
+          ++loads;
+          cur = I;
+        }
         next_tile();
       }
       if (!ok) *w.flag = 2;
+      // copies in flight land before the block ends
+      for (int s = 0; s < kSlices && loads > 0; ++s) wait_phase(&bar.full_a[s], (uint32_t)(loads - 1) & 1u);
+      for (int b = 0; b < 2; ++b)
+        if (it > b) wait_phase(&bar.full_b[b], (uint32_t)((it - b - 1) >> 1) & 1u);
     }
   } else if (warp == kEpiWarps) {
     // The whole warp runs the loop and one elected lane issues, so that the
     // descriptors stay in uniform registers: issued from a branch on the lane
-    // number, an MMA cost 110 cycles of moves, more than its operands' 68.
-    constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kNB >> 3) << 17) | ((uint32_t)(kRowBlock >> 4) << 24);
+    // number, an MMA cost 110 cycles of moves.
+    constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kRowBlock >> 4) << 24);
     const uint64_t a0 = desc_sw128(tc::smem_addr(A)), b0 = desc_sw128(tc::smem_addr(B));
-    int cur = -1;
-    uint32_t pa = 0;
+    int cur = -1, loads = 0;
     bool ok = true;
-    for (int t = t0; t < t1 && ok; ++t) {
-      const int it = t - t0, buf = it & 1;
-      if (I != cur) {
-        ok = wait_phase(&bar.full_a, pa);
-        pa ^= 1u;
-        cur = I;
-      }
-      ok = wait_phase(&bar.full_b[buf], (uint32_t)(it >> 1) & 1u) && ok;
-      ok = __all_sync(0xffffffffu, ok);
+    for (int it = 0; it < t1 - t0 && ok; ++it) {
+      const int buf = it & 1;
+      const uint32_t before = (uint32_t)(it - 1) & 1u;
+      const bool rows = I != cur;
+      loads += rows;
+      cur = I;
+      ok = wait_phase(&bar.full_b[buf], (uint32_t)(it >> 1) & 1u);
       uint64_t at = a0, bt = b0 + (uint32_t)(buf * (kBBytes >> 4));
-      asm volatile("" : "+l"(at), "+l"(bt));  // or all 136 descriptors are kept across tiles
+      asm volatile("" : "+l"(at), "+l"(bt));  // or all descriptors are kept across tiles
 #pragma unroll
-      for (int g = kGroups - 1; g >= 0; --g) {
-        if (it > 0) ok = wait_phase(&bar.drained[g], (uint32_t)(it - 1) & 1u) && ok;
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc::fence_after();
-        if (elect_one()) {
-          constexpr int kLast = kSlices - 1;
-          const int s0 = g > kLast ? g - kLast : 0, s1 = g < kLast ? g : kLast;
+      for (int s = 0; s < kSlices; ++s) {
+        if (rows) ok = wait_phase(&bar.full_a[s], (uint32_t)(loads - 1) & 1u) && ok;
+        const int slices = min(kSlices, kGroups - s);  // of the columns: t = 0 .. slices - 1
 #pragma unroll
-          for (int s = s0; s <= s1; ++s) {
-#pragma unroll
-            for (int q = 0; q < kNB / 16; ++q)  // 32 bytes along K inside the swizzled rows
-              mma_f16(tm + g * kNB, at + (uint32_t)(s * (kSliceBytes >> 4) + 2 * q),
-                      bt + (uint32_t)((g - s) * (kSliceBytes >> 5) + 2 * q), kIdesc, s > s0 || q > 0);
+        for (int t = 0; t < slices;) {
+          // S_7 begins with slices 1 and 6, which take an MMA of their own
+          const int c = min(s == 1 && t < 6 ? 6 - t : slices - t, 4);
+          const bool begin = s == 0 || (s == 1 && t == 6);
+          if (begin && it > 0) {
+            for (int g = s + t; g < s + t + c; ++g) ok = wait_phase(&bar.drained[g], before) && ok;
           }
-          tc::commit(&bar.done[g]);
-          if (g == 0) tc::commit(&bar.free_b[buf]);
+          ok = __all_sync(0xffffffffu, ok);
+          if (ok) {
+            tc::fence_after();
+            if (elect_one()) {
+#pragma unroll
+              for (int q = 0; q < kNB / 16; ++q)  // 32 bytes along K inside the swizzled rows
+                mma_f16(tm + (s + t) * kNB, at + (uint32_t)(s * (kSliceBytes >> 4) + 2 * q),
+                        bt + (uint32_t)(t * (kSliceBytes >> 5) + 2 * q),
+                        kIdesc | ((uint32_t)(c * (kNB >> 3)) << 17), !begin || q > 0);
+            }
+            __syncwarp();
+          }
+          t += c;
+        }
+        if (ok && elect_one()) {
+          tc::commit(&bar.done[s]);
+          if (s == kSlices - 1) {
+            tc::commit(&bar.done[kGroups - 1]);
+            tc::commit(&bar.free_b[buf]);
+          }
         }
         __syncwarp();
       }
@@ -725,16 +763,11 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
     }
     __syncwarp();
     wait_phase(&bar.last, 0);
-    if (!ok) {  // and so do copies: wait for each buffer's next completion
-      wait_phase(&bar.full_b[0], 0);
-      wait_phase(&bar.full_b[1], 0);
-    }
   } else {
     const int row = 32 * (warp & 3) + lane, c0 = kEpiCols * (warp >> 2);
     const uint32_t taddr = tm + ((uint32_t)(32 * (warp & 3)) << 16) + c0;
     bool ok = true;
-    for (int t = t0; t < t1 && ok; ++t) {
-      const uint32_t ph = (uint32_t)(t - t0) & 1u;
+    for (int it = 0; it < t1 - t0 && ok; ++it) {
       const int r = I * kRowBlock + row, cb = J * kNB + c0;
       double* const p0 = a + r + cb * ld;
       // entries of the lower triangle: this thread's column c exists when cb + c <= r
@@ -752,9 +785,10 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
           acc[c] = f;
         }
       }
+      unsigned top[kEpiCols];  // S_0 and S_1's part of the upper words
 #pragma unroll
-      for (int g = kGroups - 1; g >= 0; --g) {
-        ok = wait_phase(&bar.done[g], ph) && ok;
+      for (int g = 0; g < kGroups; ++g) {
+        ok = wait_phase(&bar.done[g], (uint32_t)it & 1u) && ok;
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc::fence_after();
@@ -767,11 +801,12 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
         if (lane == 0) arrive(&bar.drained[g]);
 #pragma unroll
         for (int c = 0; c < kEpiCols; ++c) {
-          const int S = __float2int_rn(__uint_as_float(v[c]));
-          if (g == 7) acc[c] -= (S + (1 << 14)) >> 15;
-          else if (g == 6) acc[c] -= (S + (1 << 5)) >> 6;
-          else if (g <= 1) acc[c] -= (long long)S << (48 - 9 * g);
-          else acc[c] = mad_wide(S, -(1 << (48 - 9 * g)), acc[c]);
+          const float S = __uint_as_float(v[c]);
+          if (g == 0) top[c] = __float_as_uint(S + kMagic) << 16;  // |S_0| <= 2^18
+          else if (g == 1) top[c] += __float_as_uint(S + kMagic) << 7;  // <= 2^21
+          else if (g >= 6) acc[c] -= __float_as_uint(fmaf(S, g == 6 ? 0x1p-6f : 0x1p-15f, kMagic));
+          else acc[c] = mad_wide(__float2int_rn(S), -(1 << (48 - 9 * g)), acc[c]);
+          if (g == 1) acc[c] += kMagicSum - ((unsigned long long)top[c] << 32);
         }
       }
       if (ok) {
@@ -837,7 +872,7 @@ cudaError_t launch_chained(void (*kernel)(P...), int64_t grid, int block, size_t
 
 // Shared memory beyond 48 KB: opted in once per device.
 cudaError_t set_chol_smem() {
-  static bool done[64] = {false};
+  static std::atomic<bool> done[64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -873,7 +908,8 @@ cudaError_t launch_loglik_fixed(double* a, int64_t n, int64_t ld, const double* 
     const int64_t below = n - (k + 1) * kNB;  // rows below the panel
     const bool wide = below > (sms - 8) * solve_rows(4);  // a few blocks stay for the substitution
     const int rows = solve_rows(wide ? 5 : 4);
-    const int row_blocks = below > 0 ? (int)((below + rows - 1) / rows) : 1;
+    // the last one has no rows of its own and writes the diagonal tile
+    const int row_blocks = 1 + (below > 0 ? (int)((below + rows - 1) / rows) : 0);
     const int extra = k == 0 ? 0 : k == 1 ? 1 : 1 + (int)((n - k * kNB + 255) / 256);
     const auto panel = k == 0 ? (wide ? chol_panel_kernel<true, 5> : chol_panel_kernel<true, 4>)
                               : (wide ? chol_panel_kernel<false, 5> : chol_panel_kernel<false, 4>);
