@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_des
                                                              const int64_t* __restrict__ sizes,
                                                              int count, BatchInstance* __restrict__ inst,
                                                              unsigned long long* __restrict__ next) {
+  asm volatile("griddepcontrol.launch_dependents;");
   const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
   if (k == 0) *next = 0ull;
   if (k >= count) return;
@@ -80,6 +81,7 @@ template <bool F32>
 __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
     const BatchInstance* __restrict__ inst, unsigned char* __restrict__ tables) {
   __shared__ TabBuildSmem sm;
+  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
   const BatchInstance& b = inst[blockIdx.y];
   if (!b.table) return;
   const MaternParams mp = b.mp;
@@ -97,6 +99,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
   __shared__ BatchInstance cur;
   __shared__ int64_t item;
   int k = -1;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   while (true) {
     __syncthreads();  // shared data of the previous round is no longer read
     if (threadIdx.x == 0) item = (int64_t)atomicAdd(next, (unsigned long long)chunk);
@@ -148,14 +151,14 @@ int tile_width(int64_t ntiles) {
   return ntiles < (int64_t)current_sm_count() * 4 ? kTabTile / 4 : kTabTile;
 }
 
-// Launches a writer so that it may be scheduled while the table's kernel before
-// it still runs (it waits for that kernel's end itself): the launch's latency,
-// about 3 us, is hidden.
+// Launches a kernel so that it may be scheduled while the one before it still
+// runs (it waits for that kernel's end itself): the launch's latency, about 3 us,
+// is hidden (batches of 3: 77.5 -> 70.9 us in FP32, 90.9 -> 86.7 in FP64).
 template <typename... P, typename... A>
-cudaError_t launch_writer(void (*kernel)(P...), unsigned grid, cudaStream_t s, A... args) {
+cudaError_t launch_next(void (*kernel)(P...), dim3 grid, int block, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(256);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block);
   cfg.stream = s;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -163,6 +166,11 @@ cudaError_t launch_writer(void (*kernel)(P...), unsigned grid, cudaStream_t s, A
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_writer(void (*kernel)(P...), unsigned grid, cudaStream_t s, A... args) {
+  return launch_next(kernel, dim3(grid), 256, s, args...);
 }
 
 template <bool F32>
@@ -241,18 +249,12 @@ cudaError_t launch_batched_table_t(const BatchTable& b, int64_t limit, int warps
   // The instances' tables in one wave of blocks; at least four each, so that the
   // node weights, once per block, stay a small part of it.
   const int sms = current_sm_count(), share = b.count < sms / 4 ? sms / b.count : 4;
-  batched_table_kernel<F32><<<dim3((unsigned)share, (unsigned)b.count), kTabThreads, 0, s>>>(
-      (const BatchInstance*)b.instances, (unsigned char*)b.tables);
-  const int grid = current_sm_count() * ctas_per_sm;
-  if (warps == 4)
-    matern_batched_table_kernel<F32, OutT, 4><<<grid, 128, 0, s>>>(
-        (const BatchInstance*)b.instances, b.count, b.prefix, limit, b.next, chunk,
-        (const unsigned char*)b.tables);
-  else
-    matern_batched_table_kernel<F32, OutT, 8><<<grid, 256, 0, s>>>(
-        (const BatchInstance*)b.instances, b.count, b.prefix, limit, b.next, chunk,
-        (const unsigned char*)b.tables);
-  return cudaGetLastError();
+  const cudaError_t e = launch_next(batched_table_kernel<F32>, dim3((unsigned)share, (unsigned)b.count),
+                                    kTabThreads, s, (const BatchInstance*)b.instances, (unsigned char*)b.tables);
+  if (e != cudaSuccess) return e;
+  return launch_next(warps == 4 ? matern_batched_table_kernel<F32, OutT, 4> : matern_batched_table_kernel<F32, OutT, 8>,
+                     dim3((unsigned)(sms * ctas_per_sm)), warps * 32, s, (const BatchInstance*)b.instances, b.count,
+                     b.prefix, limit, b.next, chunk, (const unsigned char*)b.tables);
 }
 
 }  // namespace
@@ -262,6 +264,8 @@ cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* desc
                                  cudaStream_t s) {
   batched_params_kernel<<<(unsigned)((b.count + 127) / 128), 128, 0, s>>>(
       descs, b.sizes, b.count, (BatchInstance*)b.instances, b.next);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   if (f32) return launch_batched_table_t<true, float>(b, limit, warps, ctas_per_sm, chunk, s);
   if (out_t == BK_F32) return launch_batched_table_t<false, float>(b, limit, warps, ctas_per_sm, chunk, s);
   return launch_batched_table_t<false, double>(b, limit, warps, ctas_per_sm, chunk, s);
