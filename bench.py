@@ -34,25 +34,11 @@ METRIC = "K_ν evals/s, Matérn entries/s (1 GB300): plain FP64 vs learned/FP32,
 N_LOC, BETA, SIGMA2, NUS, SEED = 20_000, 0.1, 1.0, (0.5, 1.5, 2.3), 2
 WORKLOAD = "matern_jittered_grid_n20000_beta0.1_nu{0.5,1.5,2.3}_fp64"
 
-# FP64 work model of the plain form in FP64 arithmetic operations (one per
-# thread and DFMA/DADD/DMUL): 2 per quadrature node of the common loop (the
-# summing FMA and the three-term recurrence of x cosh t; the node's
-# exponential, the factor e^{nu t} in its exponent and the geometric factor
-# 1 + e^{-2 nu t} run on the integer pipe; windows outside that loop's
-# conditions take 9 and are counted at 2), per FP64 peak Newton iteration and
-# per FP64 window-end Newton iteration (these run only for windows the check
-# rejects, or outside the FP32 search region), and a fixed part per Matern
-# entry (the distance, r^2 times the matrix's constant, set-ups, the
-# exponent step K nu h, the end terms' scaling, the exponent's FMAs; the
-# square root, log x and the final exponential run on the integer pipe).  The
-# fixed part is ncu's executed DFMA + DADD + DMUL per evaluation minus 2 x
-# nodes per evaluation on the n = 6000 case of the same kernel
-# (--profile-case plain_nus: 14.89 for each of nu = 0.5, 1.5, 2.3).
-# The FP32 Newton iterations that place the window and the FP32 window check
-# run on the FP32/MUFU pipes and are not counted.
-OPS_NODE, OPS_PEAK_IT, OPS_WIN_IT, OPS_ENTRY_FIXED = 2, 54, 31, 14.9
-# Kernels per bk_matern_tile call of the plain form: the per-launch table of
-# e^{-2 nu h} on the quantised steps, then the symmetric tile writer.
+# Rate of a plain device-to-device copy on a GB300 (read plus write bytes), the
+# denominator for the matrix writers: a matrix costs at least its own bytes.
+HBM_COPY_GBS = 6666.6
+# Kernels per bk_matern_tile call of the plain form: the call's table of M(r^2),
+# then the symmetric tile writer that reads it.
 LAUNCHES_PER_MATRIX = 2
 # FP64 pipe peak from the unit count and clock: 152 SMs x 2 DFMA/clk x 2.07 GHz
 # (1.26 TFLOP/s counting an FMA as two FLOPs).
@@ -168,9 +154,10 @@ class ClockSampler:
                 "sm_max_mhz": max(r[1] for r in rows), "reasons": reasons, "samples": len(rows)}
 
 
-KERNEL_SOURCES = ("bk_plain.cu", "bk_math64.cuh", "bk_math32.cuh", "bk_forms.cuh", "bk_tiles.cuh",
-                  "bk_matern_common.cuh", "bk_exp2_table.inc", "bk_cosh_table.inc")
-# The FP32 forms' kernels (single matrix, bare evaluations, batched, learned).
+KERNEL_SOURCES = ("bk_entry_table.cu", "bk_entry_table.cuh", "bk_math64.cuh", "bk_math32.cuh",
+                  "bk_forms.cuh", "bk_tiles.cuh", "bk_matern_common.cuh", "bk_exp2_table.inc",
+                  "bk_tau_table.inc")
+# The FP32 forms' kernels that evaluate every entry by itself (bare evaluations).
 FP32_SOURCES = ("bk_math64.cuh", "bk_math32.cuh", "bk_forms.cuh", "bk_tiles.cuh",
                 "bk_matern_common.cuh", "bk_peak_table.inc", "bk_fp32.cu", "bk_learned.cu",
                 "bk_batched.cu")
@@ -299,7 +286,7 @@ def config(n):
             "n": n, "sigma2": SIGMA2, "beta": BETA, "nu": list(NUS), "locations": "jittered grid, "
             "Morton order, seed 2", "output_bytes_per_matrix": n * n * 8,
             "l2": "inputs larger than L2: each step writes 3 x n^2 x 8 B of output; no flush",
-            "form": "plain FP64 (peak search + eps=2^-52 window + strip-bound node count)",
+            "form": "plain FP64 (entries from the call's table of M(r^2))",
             "parallelism": "one process per GPU, independent matrices (weak)"}
 
 
@@ -355,6 +342,15 @@ def issue_roofline(key, kernel, launch_s, evals):
     return out
 
 
+def write_roofline(kernel, launch_s, nbytes):
+    """Roofline of a matrix writer against its output's bytes."""
+    achieved = nbytes / launch_s / 1e9
+    return {"bound": "memory", "kernel": kernel, "unit": "GB/s", "achieved": achieved,
+            "peak": HBM_COPY_GBS, "frac": achieved / HBM_COPY_GBS,
+            "peak_source": "measured: device-to-device copy, read + write bytes",
+            "algorithmic_bytes_per_launch": nbytes}
+
+
 def measure_forms(bk, inputs, dev, stream, args, plain_rate):
     """Throughput, roofline, counters and output samples of the other forms
     (outside the headline timing).  The samples are checked against the
@@ -388,8 +384,8 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
     res["fp32_matern"] = {
         "workload": f"C3: n={n3} jittered grid, beta={beta3}, nu={nu3:.4f} (U(0.3,3.5), seed 5), "
                     "FP32 out", "value": n3 * n3 / t, "unit": "entries/s", "ms": 1e3 * t,
-        "counters": cs, "roofline": issue_roofline("fp32_matern", "matern_sym_kernel<FormF32, float>",
-                                                   t, cs["evals"])}
+        "counters": cs, "roofline": write_roofline("matern_table_kernel<true, float, true>", t,
+                                                   4 * n3 * n3)}
     sample_matrix("fp32_matern", o32, L3h, 1.0, beta3, nu3, 1_000_000, 6, 0.01)
 
     # -- C5 matrix: learned window vs searched window vs plain FP64, n = 40,000, beta = 0.1,
@@ -415,8 +411,7 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
         "plain_fp64_value": n5 * n5 / t_p, "unit": "entries/s",
         "learned_over_plain": t_p / t_l, "learned_over_fp32_search": t_s / t_l,
         "counters": cl, "fallback_rate": cl["fallback_rate"],
-        "roofline": issue_roofline("learned_matern", "matern_sym_kernel<FormF32Learned, float>",
-                                   t_l, cl["evals"])}
+        "roofline": write_roofline("matern_table_kernel<true, float, true>", t_l, 4 * n5 * n5)}
     del L3
     torch.cuda.empty_cache()
 
@@ -501,10 +496,8 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
                        2 if name == "fp64" else 5)
             bres[name]["static_value"] = entries / ts
         if name != "fp64":
-            key = "batched_" + name
-            kern = ("matern_batched_kernel<FormF32Learned, float>" if form_opts
-                    else "matern_batched_kernel<FormF32, float>")
-            bres[name]["roofline"] = issue_roofline(key, kern, tb, cbs["evals"])
+            bres[name]["roofline"] = write_roofline("matern_batched_table_kernel<true, float>", tb,
+                                                    4 * entries)
         if name == "learned_fp32":
             bres[name]["fallback_rate"] = cbs["fallback_rate"]
             for k, (inst, o) in enumerate(zip(insts, outs)):
@@ -546,7 +539,7 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
     del o2, L2, refs
     torch.cuda.empty_cache()
 
-    # -- downstream Gaussian log-likelihood (blocked FP64 Cholesky) on the n = 4,000 and
+    # -- downstream Gaussian log-likelihood (fixed-point Cholesky) on the n = 4,000 and
     # n = 8,000 Matern matrices of the Cholesky checks (jittered grid seed 3, beta 0.1, nu 0.5)
     ll = {"unit": "s", "workload": "jittered grid (seed 3), sigma2 1, beta 0.1, nu 0.5, "
                                    "z ~ N(0, 1) (seed 5): matrix generation + log-likelihood"}
@@ -562,7 +555,7 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
         t_ll = _time(lambda: bk.bk_gaussian_loglik(ml, zl, y=yl, out=outl), stream, 1)
         bk.bk_matern_tile(Ll, SIGMA2, BETA, 0.5, out=ml)  # the last call factored ml in place
         ll[f"n{nl}"] = {"matern_s": t_gen, "loglik_s": t_ll,
-                        "cholesky_fp64_tflops": nl ** 3 / 3 / t_ll / 1e12,
+                        "cholesky_tflops": nl ** 3 / 3 / t_ll / 1e12,
                         "loglik": float(bk.bk_gaussian_loglik(ml, zl, y=yl, out=outl)[0])}
         del Ll, zl, ml, yl
         torch.cuda.empty_cache()
@@ -847,8 +840,8 @@ def main():
     out = torch.empty((n, n), dtype=torch.float64, device=dev)
     stream = torch.cuda.current_stream()
 
-    # -- work accounting pass (untimed): nodes / iterations per launch
-    flop_per_launch = []
+    # -- accounting pass (untimed): counters are kept by the entries' own evaluation
+    # (window and quadrature), which the tables replace and fall back to
     work = []
     fails = fallbacks = evals_counted = 0
     for nu in NUS:
@@ -862,8 +855,6 @@ def main():
                      "iters_per_entry": float(c[bk.BK_CTR_ITERS] / max(1, c[bk.BK_CTR_EVALS])),
                      "peak_iters_per_entry": float(c[bk.BK_CTR_PEAK_ITERS]
                                                    / max(1, c[bk.BK_CTR_EVALS]))})
-        flop_per_launch.append(OPS_NODE * c[bk.BK_CTR_NODES] + OPS_PEAK_IT * c[bk.BK_CTR_PEAK_ITERS]
-                               + OPS_WIN_IT * c[bk.BK_CTR_ITERS] + OPS_ENTRY_FIXED * c[bk.BK_CTR_EVALS])
     torch.cuda.synchronize()
 
     def step(ev=None):
@@ -911,17 +902,9 @@ def main():
 
     # -- roofline of the dominant kernel (the symmetric FP64 tile writer)
     mean_launch_s = statistics.mean(statistics.mean(v) for v in launch_ms) / 1e3
-    flop_mean = float(np.mean(flop_per_launch))
-    achieved = flop_mean / mean_launch_s / 1e9
-    roofline = {"bound": "alu", "kernel": "matern_sym_kernel<FormF64T<false>, double>",
-                "achieved": achieved, "peak": FP64_PEAK_GOPS, "unit": "FP64 Gop/s",
-                "frac": achieved / FP64_PEAK_GOPS,
-                "peak_source": "derived: 152 SMs x 2 FP64 ops/clk x 2.07 GHz (of derived)",
-                "traffic": profiled_traffic(n),
-                "pipes_ncu": profiled_pipes(),
-                "algorithmic_fp64_ops_per_launch": flop_mean,
-                "algorithmic_bytes_per_launch": n * n * 8 + 16 * n,
-                "work": work}
+    roofline = write_roofline("matern_table_kernel<false, double, true>", mean_launch_s, 8 * n * n)
+    roofline.update({"limited_by": "record loads (L1) and integer pipes", "traffic": profiled_traffic(n),
+                     "pipes_ncu": profiled_pipes(), "direct_evaluation": work})
 
     # -- pipe probes (context for the peak)
     sink = torch.empty(152 * 8 * 256, dtype=torch.float64, device=dev)
@@ -937,14 +920,8 @@ def main():
         torch.cuda.synchronize()
         mult = 2 if kind in (0, 1) else 1  # an FMA counts 2 FLOPs
         probe[name] = ops * mult / (a.elapsed_time(b) / 1e3) / 1e12
-    # Measured context for the derived peaks: the DFMA probe's operations/s (a
-    # stream of independent FP64 FMAs reaches ~0.8 of the unit-count rate,
-    # below the FP64 operations/s the tile writer itself sustains, so it is no
-    # ceiling), and the FFMA probe's thread instructions/s (the issue limit).
-    dfma_gops = probe["fp64_fma_tflops"] / 2 * 1e3
+    # The FFMA probe's thread instructions/s: the measured issue limit.
     issue_ginst = probe["fp32_fma_tflops"] / 2 * 1e3
-    roofline.update({"peak_measured": dfma_gops, "frac_measured": achieved / dfma_gops,
-                     "peak_measured_source": "bk_probe_pipe kind 0 (independent DFMA chains)"})
 
     # -- secondary: bare K_nu evaluation, 100,000 pairs (x log-uniform in [1e-3,140], nu in [0.05,10])
     xh, nh = inputs.kv_pairs(100_000, seed=1)
@@ -985,9 +962,7 @@ def main():
         forms, samples = measure_forms(bk, inputs, dev, stream, args, value)
 
     if forms is not None:
-        for r in ([forms["fp32_matern"]["roofline"], forms["learned_matern"]["roofline"],
-                   forms["learned_eval"]["roofline"], forms["learned_eval"]["fp32_search_roofline"]]
-                  + [forms["batched"][k]["roofline"] for k in ("fp32", "learned_fp32")]):
+        for r in (forms["learned_eval"]["roofline"], forms["learned_eval"]["fp32_search_roofline"]):
             r["peak_measured"] = issue_ginst
             r["peak_measured_source"] = "bk_probe_pipe kind 1 (independent FFMA chains)"
             r["frac_measured"] = r["achieved"] / issue_ginst if r["achieved"] else None
