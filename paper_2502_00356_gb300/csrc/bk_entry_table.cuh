@@ -171,7 +171,9 @@ __device__ __forceinline__ int tab_octave(int k, const MaternParams& mp) {
 // records.  The FP64 pipe bounds it (an operation of one warp takes 17 cycles of
 // the SM), so the exponentials run on the integer pipe (exp2s_int), every SM takes
 // part, a block's intervals grid-strided so that each gets the same share of
-// costly ones, and warps without an interval do nothing.  Small matrices leave most
+// costly ones, warps without an interval do nothing, one thread computes 1/beta^2
+// for all, and a sum over lanes costs one addition a step for both values (n = 777:
+// 28.9 us with 1/beta^2 in every thread and two additions, 26.6 so).  Small matrices leave most
 // intervals out (r2_max): then latency bounds it, and 16 or 32 lanes share one
 // (n = 777: eight took 21,000 cycles for the sums).
 constexpr int kTabThreads = 1024;
@@ -179,6 +181,7 @@ constexpr int kTabGroups = kTabThreads / 8;  // at most
 struct TabBuildSmem {
   double v[kTabNodes], w[kTabNodes], w2[kTabNodes];
   double f0[kTabGroups], f1[kTabGroups];
+  double b2, b2lo;  // 1/beta^2
   float box[kTabThreads / 64][4];
 };
 
@@ -376,12 +379,16 @@ __device__ __forceinline__ void tab_build_block(TabBuildSmem& sm, const MaternPa
   static_assert(kTabNodes <= kTabThreads - kTabScanThreads, "nodes and scan side by side");
   if (threadIdx.x < kTabThreads - kTabScanThreads) tab_nodes(sm, mp.nu, mp.log_pref);
   else if (scan) tab_scan(sm.box, locs1, m_locs, locs2, n_locs);
+  if (threadIdx.x == kTabThreads - 1) {
+    // x^2 = s_ref/beta^2, with the rounding of 1/beta and of its square taken back
+    const double ib = mp.inv_beta, b2 = ib * ib;
+    sm.b2 = b2;
+    sm.b2lo = fma(ib, ib, -b2) + 2.0 * ib * (fma(-ib, mp.beta, 1.0) * ib);
+  }
   __syncthreads();
   const double r2_max = scan ? tab_r2_bound(sm.box) : kInf;
   const unsigned e0 = tab_first_binade(mp.inv_beta);
-  // x^2 = s_ref/beta^2, with the rounding of 1/beta and of its square taken back
-  const double ib = mp.inv_beta, b2 = ib * ib;
-  const double b2lo = fma(ib, ib, -b2) + 2.0 * ib * (fma(-ib, mp.beta, 1.0) * ib);
+  const double ib = mp.inv_beta, b2 = sm.b2, b2lo = sm.b2lo;
   const float nuf = f32_trunc(mp.nu);
   if (block == blocks - 1) {
     if (threadIdx.x < L::kExtra) {
@@ -438,14 +445,15 @@ __device__ __forceinline__ void tab_build_block(TabBuildSmem& sm, const MaternPa
         }
       }
       const unsigned mask = lanes == 32 ? 0xffffffffu : ((1u << lanes) - 1u) << (threadIdx.x & 31 & -lanes);
-      for (int d = 1; d < lanes; d <<= 1) {
-        f0 += __shfl_xor_sync(mask, f0, d);
-        f1 += __shfl_xor_sync(mask, f1, d);
-      }
-      if (lane == 0) {
+      // half of the lanes go on with F_nu, half with F_{nu-1}
+      const int half = lanes >> 1;
+      const bool second = (lane & half) != 0;
+      double f = second ? f1 : f0;
+      f += __shfl_xor_sync(mask, second ? f0 : f1, half);
+      for (int d = 1; d < half; d <<= 1) f += __shfl_xor_sync(mask, f, d);
+      if ((lane & (half - 1)) == 0) {
         const double h = step == 1 ? 1.0 : step == 2 ? 2.0 : step == 3 ? 3.0 : 4.0;
-        sm.f0[k] = h * f0;
-        sm.f1[k] = h * f1;
+        (second ? sm.f1 : sm.f0)[k] = h * f;
       }
     }
     __syncthreads();
