@@ -290,7 +290,9 @@ __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld,
 // rows are solved at no extra time, without a barrier.  The group's update (rank
 // 8) of the next group's columns happens in the solving warps' registers; the
 // other warps apply it to the columns after those while the solving warps are at
-// the next group: one barrier a group.  Four warps carry 96 rows, the tile's 56 and
+// the next group: one barrier a group.  The factored 8 x 8 blocks have a place of
+// their own: all solving warps read a group's block between the same two barriers
+// as one of them has its factor, so nothing is written where they read.  Four warps carry 96 rows, the tile's 56 and
 // 32 below it; where more are needed to fill one wave of the SMs a fifth warp
 // takes 64 below it, which shares a scheduler and slows the chain.  A product
 // costs three wide multiply-adds of 8 cycles a warp and scheduler (an FP64 FMA 64),
@@ -302,6 +304,7 @@ constexpr int kFollow = 24;
 constexpr int solve_rows(int solve) { return solve == 4 ? 32 : 64; }  // rows below the tile
 struct PanelSmem {
   long long S[2 * kNB][kNB + 1];   // two's complement before, limbs after a column is done
+  long long D[kNB][8];             // the diagonal 8 x 8 blocks' factors (limbs), row by row
   int scale[2 * kNB];
   int bad;
 };
@@ -441,8 +444,10 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
       }
       if (lane >= 8 ? follow >= c0 + 8 : warp == kSolve - 1) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-          if (lane >= 8 || c <= lane) sm.S[row][c0 + c] = v[c];
+        for (int c = 0; c < 8; ++c) {
+          if (lane >= 8) sm.S[row][c0 + c] = v[c];
+          else if (c <= lane) sm.D[row][c] = v[c];
+        }
       }
       if (bad && lane == 0) sm.bad = 1;
     } else if (c0 > 0) {
@@ -479,7 +484,10 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
     for (int e = tid; e < kNB * kNB; e += kPanelThreads) {
       const int r = e & 63, c = e >> 6;
       double v = r == c ? 1.0 : 0.0;
-      if (r < b && c <= r) v = bad ? qnan() : from_fixed(value(as_limbs(sm.S[r][c])), sm.scale[r]);
+      if (r < b && c <= r) {
+        const long long x = c >= (r & ~7) ? sm.D[r][c & 7] : sm.S[r][c];
+        v = bad ? qnan() : from_fixed(value(as_limbs(x)), sm.scale[r]);
+      }
       w.diag[(k & 1) * (kNB * kNB) + e] = v;
     }
   }
