@@ -455,9 +455,11 @@ bk_status bk_gaussian_loglik(double* a, int64_t n, int64_t ld, const double* z, 
  * bits of sqrt(a_ii a_jj)): the trailing updates as exact digit products on the
  * tensor cores (tcgen05), the panels on the integer pipe.  Its rounding is
  * below that of FP64 relative to sqrt(a_ii a_jj); entries of L far below their
- * row's norm carry that absolute accuracy.  A matrix with |a_ij| >= 2
- * sqrt(a_ii a_jj) or a non-finite entry counts as not positive definite.  Two
- * launches per 64 rows.  d_work == NULL or too small: bk_gaussian_loglik. */
+ * row's norm carry that absolute accuracy.  A matrix with an entry that is not
+ * finite, or that reaches 2^{s_i + s_j} (2^{2 s_i} the power of four above a_ii,
+ * so between 1 and 4 times sqrt(a_ii a_jj)), counts as not positive definite, as
+ * does one with a pivot <= 0 or with a row of L longer than its diagonal entry
+ * allows.  Two launches per 64 rows.  d_work == NULL or too small: bk_gaussian_loglik. */
 size_t bk_gaussian_loglik_workspace(int64_t n);
 bk_status bk_gaussian_loglik_ws(double* a, int64_t n, int64_t ld, const double* z, double* y,
                                 double* out, const bk_opts* opts, void* d_work, size_t work_bytes,

@@ -13,8 +13,13 @@
 // The lower triangle is converted in place and factored as integers in units
 // of 2^-60; every finished panel is written back as FP64.  Rounding is 2^-60 to
 // 2^-57 of sqrt(a_ii a_jj) a step, against FP64's 2^-53 of the numbers at hand.
-// An input outside those bounds, or a pivot that is not positive, means the
-// matrix is not positive definite.
+// An input outside those bounds, a pivot that is not positive, or a row of L
+// longer than its diagonal allows means that the matrix is not positive definite.
+// All three are tested, so that no integer wraps around unnoticed: before a column
+// is scaled, |v| < 2^60 sqrt(D 2^-60) for what stands below its pivot D (within a
+// factor of 4; the products hold that); the sum of the squares of a panel's part of
+// a row (within 1/16); and the sign of what an update leaves of the diagonal.  Every
+// number of an accepted matrix then stays below 2^62.
 //
 // Digits.  x = sum_s d_s 2^{54 - 9 s}, s = 0 .. 6, d_s in [-256, 255] (|d_0| <=
 // 64): exact.  A product of two rows is sum_g 2^{48 - 9 g} S_g in units of 2^-60,
@@ -185,11 +190,25 @@ __device__ __forceinline__ long long rsqrt_fixed(long long D, int& t) {
   return ((long long)Y << 37) + (p >> 9);
 }
 
-// (v 2^t) rho / 2^60, v of magnitude below 2^{60 - t}.
+// (v 2^t) rho / 2^60, v of magnitude below 2^{61 - t} (too_large).
 __device__ __forceinline__ long long mul_rho(long long v, int t, Limbs rho) {
   Acc a;
   a.add(limbs(v << t), rho);
   return a.sum();
+}
+
+// Whether |v| >= 2^{61 - t} (-2^{61 - t} itself passes); t <= 30.
+__device__ __forceinline__ bool too_large(long long v, int t) {
+  if (t > 29) return (unsigned long long)((v >> 31) + 1) > 1ULL;  // D below 4 units
+  return (unsigned)(((int)(v >> 32) >> (29 - t)) + 1) > 1u;
+}
+
+// The sum of (x 2^-50)^2 over columns of a row: at most (2^10)^2 in exact numbers,
+// and less than 2^14 + 64 more by truncation; |x| < 2^62, so that 64 squares fit.
+constexpr unsigned kRowSquares = (1u << 20) + (1u << 15);
+__device__ __forceinline__ unsigned add_square(unsigned sum, Limbs x) {
+  const int h = x.h >> 18;
+  return sum + (unsigned)(h * h);
 }
 
 // Scales, y = z, the flag.
@@ -398,6 +417,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
   __syncthreads();
   const int groups = own > 32 ? 4 : own > 0 ? 3 : 2;  // row groups of 32
   const int follow = 8 + kFollow * warp + lane - 8;   // a solving lane's row (lanes 8 .. 31)
+  unsigned squares = 0;                               // of that row
   for (int c0 = 0; c0 < kNB; c0 += 8) {
     // solving warps whose rows are all done (the tile's first ones) join the others
     const int retired = min(c0 / kFollow, kSolve - 1);
@@ -421,7 +441,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
           v[j] -= acc.sum();
         }
       }
-      bool bad = false;
+      bool bad = false, over = false;
+      if (lane < 8) squares = 0;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         long long D = shfl64(v[c], c);
@@ -431,7 +452,10 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
         }
         int t;
         const Limbs rho = limbs(rsqrt_fixed(D, t));
+        const bool below = lane > c;
+        over = (below && too_large(v[c], t)) || over;
         const Limbs x = limbs(mul_rho(v[c], t, rho));
+        if (below) squares = add_square(squares, x);
         v[c] = raw_limbs(x);
 #pragma unroll
         for (int j = c + 1; j < 8; ++j) {
@@ -442,6 +466,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
           v[j] -= p.sum();
         }
       }
+      // (rows above the group's block hold nothing that counts)
+      if ((lane < 8 || follow >= c0 + 8) && (over || squares > kRowSquares)) bad = true;
       if (lane >= 8 ? follow >= c0 + 8 : warp == kSolve - 1) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
@@ -449,7 +475,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
           else if (c <= lane) sm.D[row][c] = v[c];
         }
       }
-      if (bad && lane == 0) sm.bad = 1;
+      if (bad) sm.bad = 1;
     } else if (c0 > 0) {
       // the rest of the previous group's update: columns from c0 + 8 on
       const int rest = kPanelThreads / 32 - kSolve + retired, u = warp < kSolve ? warp : warp - kSolve + retired;
@@ -479,8 +505,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
     __syncthreads();
   }
   const bool bad = sm.bad != 0;
+  if (bad && tid == 0) *w.flag = 1;
   if ((int)blockIdx.x == row_blocks - 1) {
-    if (bad && tid == 0) *w.flag = 1;
     for (int e = tid; e < kNB * kNB; e += kPanelThreads) {
       const int r = e & 63, c = e >> 6;
       double v = r == c ? 1.0 : 0.0;
@@ -826,6 +852,11 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
           else acc[c] = mad_wide(__float2int_rn(S), -(1 << (48 - 9 * g)), acc[c]);
           if (g == 1) acc[c] += kMagicSum - ((unsigned long long)top[c] << 32);
         }
+      }
+      if (ok && J >= 2 * I) {  // a tile on the diagonal
+#pragma unroll
+        for (int c = 0; c < kEpiCols; ++c)
+          if (cb + c == r && r < n && acc[c] <= 0) *w.flag = 1;
       }
       if (ok) {
         p = p0;
