@@ -179,6 +179,34 @@ def _dev(t, name: str, dtype=None):
     return t
 
 
+def _empty(shape, dtype, device, stream, kept=True):
+    """torch.empty for a call on ``stream`` (None: the current stream), from
+    torch's caching allocator, so that the library allocates nothing and graph
+    capture takes it from the graph's pool.  The allocator hands a block out
+    again in the order of the stream it was allocated on, so it is allocated on
+    the stream that writes it: work that the current stream still has to do on
+    a block freed earlier is not waited for there.  ``kept``: the caller gets
+    the tensor and may use it on the current stream."""
+    torch = _torch()
+    if stream is None:
+        return torch.empty(shape, dtype=dtype, device=device)
+    if not isinstance(stream, torch.cuda.Stream):
+        handle = _stream_ptr(stream)
+        stream = (torch.cuda.ExternalStream(handle, device=device) if handle
+                  else torch.cuda.default_stream(device))
+    current = torch.cuda.current_stream(device)
+    with torch.cuda.stream(stream):
+        t = torch.empty(shape, dtype=dtype, device=device)
+    if kept and stream != current:
+        t.record_stream(current)
+    return t
+
+
+def _scratch(nbytes: int, device, stream):
+    """Device scratch of ``nbytes`` for one call on ``stream``."""
+    return _empty(max(int(nbytes), 1), _torch().uint8, device, stream, kept=False)
+
+
 def _ptr(t) -> Optional[int]:
     return None if t is None else (t.data_ptr() or None)
 
@@ -246,7 +274,7 @@ def bk_eval(x, nu, out=None, stream=None):
     if x.numel() != nu.numel():
         raise ValueError("x and nu must have the same number of elements")
     if out is None:
-        out = torch.empty_like(x)
+        out = _empty(x.shape, torch.float64, x.device, stream)
     _dev(out, "out", torch.float64)
     if out.numel() != x.numel():
         raise ValueError("out has the wrong size")
@@ -267,10 +295,10 @@ def bk_eval_ex(x, nu, out=None, log_out=None, out_dtype=None, opts: Optional[bk_
         out_dtype = out.dtype if out is not None else torch.float64
     code = _dtype_code(out_dtype)
     if out is None:
-        out = torch.empty(x.shape, dtype=out_dtype, device=x.device)
+        out = _empty(x.shape, out_dtype, x.device, stream)
     _dev(out, "out", out_dtype)
     if want_log and log_out is None:
-        log_out = torch.empty(x.shape, dtype=out_dtype, device=x.device)
+        log_out = _empty(x.shape, out_dtype, x.device, stream)
     if log_out is not None:
         _dev(log_out, "log_out", out_dtype)
     optp = ctypes.byref(opts) if opts is not None else None
@@ -308,7 +336,7 @@ def bk_eval_grad(x, nu, k=None, dk_dx=None, dk_dnu=None, opts: Optional[bk_opts]
     outs = []
     for t, name in ((k, "k"), (dk_dx, "dk_dx"), (dk_dnu, "dk_dnu")):
         if t is None:
-            t = torch.empty(x.shape, dtype=torch.float64, device=x.device)
+            t = _empty(x.shape, torch.float64, x.device, stream)
         _dev(t, name, torch.float64)
         if t.numel() != n:
             raise ValueError(f"{name} has the wrong size")
@@ -333,9 +361,9 @@ def bk_gaussian_loglik(a, z, y=None, out=None, opts: Optional[bk_opts] = None, s
     if z.numel() != n:
         raise ValueError("z must have n elements")
     if y is None:
-        y = torch.empty(n, dtype=torch.float64, device=a.device)
+        y = _empty(n, torch.float64, a.device, stream)
     if out is None:
-        out = torch.empty(3, dtype=torch.float64, device=a.device)
+        out = _empty(3, torch.float64, a.device, stream)
     _dev(y, "y", torch.float64)
     _dev(out, "out", torch.float64)
     optp = ctypes.byref(opts) if opts is not None else None
@@ -356,23 +384,6 @@ def _locs(locs, name="locs"):
 BK_COSH_TABLE_LEN = 3328
 
 
-def _scratch(nbytes: int, device, stream):
-    """Device scratch of ``nbytes`` from torch's caching allocator (so the
-    library allocates nothing and graph capture takes it from the graph's
-    pool).  Freed memory is reused in the order of the current stream; for a
-    call on another stream the allocator is told of that use."""
-    torch = _torch()
-    t = torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device=device)
-    if stream is not None:
-        if isinstance(stream, int):
-            stream = torch.cuda.ExternalStream(stream, device=device) if stream else None
-        if stream is None:
-            stream = torch.cuda.default_stream(device)
-        if stream != torch.cuda.current_stream(device):
-            t.record_stream(stream)
-    return t
-
-
 def bk_matern_tile(locs, sigma2: float, beta: float, nu: float, out=None, dtype=None,
                    opts: Optional[bk_opts] = None, stream=None):
     """Full n x n Matern matrix of SoA locations (2, n).  ``out`` is a CUDA
@@ -381,7 +392,7 @@ def bk_matern_tile(locs, sigma2: float, beta: float, nu: float, out=None, dtype=
     torch = _torch()
     n = _locs(locs)
     if out is None:
-        out = torch.empty((n, n), dtype=dtype or torch.float64, device=locs.device)
+        out = _empty((n, n), dtype or torch.float64, locs.device, stream)
     code = _dtype_code(out.dtype)
     _dev(out, "out")
     if out.dim() != 2 or out.shape[0] != n or out.shape[1] < n:
@@ -445,7 +456,7 @@ def bk_matern_tile2(locs1, locs2, sigma2: float, beta: float, nu: float, out=Non
     m = _locs(locs1, "locs1")
     n = _locs(locs2, "locs2")
     if out is None:
-        out = torch.empty((n, m), dtype=dtype or torch.float64, device=locs1.device)
+        out = _empty((n, m), dtype or torch.float64, locs1.device, stream)
     code = _dtype_code(out.dtype)
     _dev(out, "out")
     if out.dim() != 2 or out.shape[0] != n or out.shape[1] < m:
@@ -502,7 +513,7 @@ def bk_math_probe(fn, x, stream=None):
     k = MATH_PROBE_FNS[fn] if isinstance(fn, str) else int(fn)
     x = x.contiguous()
     n = x.numel()
-    out = torch.empty(2 * n if k == 4 else n, dtype=torch.float64, device=x.device)
+    out = _empty(2 * n if k == 4 else n, torch.float64, x.device, stream)
     _check(lib().bk_math_probe(k, _ptr(x), _ptr(out), n, _stream_ptr(stream)))
     return out.view(n, 2) if k == 4 else out.view(x.shape)
 
@@ -643,15 +654,15 @@ class LearnedWindow:
         """(gradient[8772], loss) of the full-batch loss over the given samples."""
         torch = _torch()
         n = x.numel()
-        g = torch.empty(N_MLP_PARAMS, dtype=torch.float32, device=x.device)
-        loss = torch.zeros(1, dtype=torch.float32, device=x.device)
+        g = _empty(N_MLP_PARAMS, torch.float32, x.device, stream)
+        loss = _empty(1, torch.float32, x.device, stream)
         _check(lib().bk_learned_grad(self.handle, _ptr(x), _ptr(nu), _ptr(labels), n, _ptr(g),
                                      _ptr(loss), _stream_ptr(stream)))
         return g, loss
 
     def infer(self, x, nu, stream=None):
         torch = _torch()
-        out = torch.empty((x.numel(), 4), dtype=torch.float32, device=x.device)
+        out = _empty((x.numel(), 4), torch.float32, x.device, stream)
         _check(lib().bk_learned_infer(self.handle, _ptr(x), _ptr(nu), _ptr(out), x.numel(),
                                       _stream_ptr(stream)))
         return out
