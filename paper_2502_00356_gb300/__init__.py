@@ -179,8 +179,8 @@ def _dev(t, name: str, dtype=None):
     return t
 
 
-def _empty(shape, dtype, device, stream, kept=True):
-    """torch.empty for a call on ``stream`` (None: the current stream), from
+def _empty(shape, dtype, device, stream, kept=True, zero=False):
+    """torch.empty (``zero``: torch.zeros) for a call on ``stream`` (None: the current stream), from
     torch's caching allocator, so that the library allocates nothing and graph
     capture takes it from the graph's pool.  The allocator hands a block out
     again in the order of the stream it was allocated on, so it is allocated on
@@ -188,15 +188,16 @@ def _empty(shape, dtype, device, stream, kept=True):
     a block freed earlier is not waited for there.  ``kept``: the caller gets
     the tensor and may use it on the current stream."""
     torch = _torch()
+    new = torch.zeros if zero else torch.empty
     if stream is None:
-        return torch.empty(shape, dtype=dtype, device=device)
+        return new(shape, dtype=dtype, device=device)
     if not isinstance(stream, torch.cuda.Stream):
         handle = _stream_ptr(stream)
         stream = (torch.cuda.ExternalStream(handle, device=device) if handle
                   else torch.cuda.default_stream(device))
     current = torch.cuda.current_stream(device)
     with torch.cuda.stream(stream):
-        t = torch.empty(shape, dtype=dtype, device=device)
+        t = new(shape, dtype=dtype, device=device)
     if kept and stream != current:
         t.record_stream(current)
     return t
@@ -655,7 +656,7 @@ class LearnedWindow:
         torch = _torch()
         n = x.numel()
         g = _empty(N_MLP_PARAMS, torch.float32, x.device, stream)
-        loss = _empty(1, torch.float32, x.device, stream)
+        loss = _empty(1, torch.float32, x.device, stream, zero=True)
         _check(lib().bk_learned_grad(self.handle, _ptr(x), _ptr(nu), _ptr(labels), n, _ptr(g),
                                      _ptr(loss), _stream_ptr(stream)))
         return g, loss
