@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(kTabThreads) entry_table_kernel(
 // do not gain from more (n = 20,000: 3 blocks 1,139, 4 1,079, 5 1,081, 6 1,142).
 template <bool F32, typename OutT, bool kSym>
 __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
-    const unsigned char* __restrict__ table, const double* __restrict__ locs1, int64_t m,
+    const unsigned char* table, const double* __restrict__ locs1, int64_t m,
     const double* __restrict__ locs2, int64_t n, const __grid_constant__ MaternParams mp,
     OutT* __restrict__ out, int64_t ld, int64_t tiles_m, int64_t col_base, int width) {
   __shared__ TabTileSmem<F32, OutT> sm;
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_des
 
 template <bool F32>
 __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
-    const BatchInstance* __restrict__ inst, unsigned char* __restrict__ tables) {
+    const BatchInstance* inst, unsigned char* __restrict__ tables) {  // (inst: not read-only, load_record)
   __shared__ TabBuildSmem sm;
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
   const BatchInstance& b = inst[blockIdx.y];
@@ -92,9 +92,9 @@ __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
 // Persistent kernel as matern_batched_kernel, in tiles of 64.
 template <bool F32, typename OutT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_kernel(
-    const BatchInstance* __restrict__ inst, int count, const int64_t* __restrict__ prefix,
+    const BatchInstance* inst, int count, const int64_t* __restrict__ prefix,
     int64_t limit, unsigned long long* __restrict__ next, int chunk,
-    const unsigned char* __restrict__ tables) {
+    const unsigned char* tables) {
   __shared__ TabTileSmem<F32, OutT> sm;
   __shared__ BatchInstance cur;
   __shared__ int64_t item;

@@ -521,6 +521,26 @@ __device__ __forceinline__ long long fix_mod(double v, int s) {
   return (long long)b < 0 ? -(long long)r : (long long)r;
 }
 
+// Loads of a table by kernels that are launched while an earlier grid may still
+// write it, which they wait for first: plain loads, as the read-only path (ld.global.nc)
+// is for memory that nothing writes while the kernel lives.  A record's address comes
+// from a word, a word's load is volatile: neither moves ahead of the wait.
+__device__ __forceinline__ uint4 load_record(const uint4* p) {
+  uint4 v;
+  asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 load_record(const float4* p) {
+  float4 v;
+  asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int load_word(const int* p) {
+  int v;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // Stages a tile's points and words; every thread of the block calls it (the caller
 // synchronises before, when sm was read, and after).  False: the tile spans
 // more than any table could use, or is not finite.
@@ -528,7 +548,7 @@ template <bool F32, int THREADS>
 __device__ __forceinline__ bool tab_stage(TabPoints<F32>& sm, const double* __restrict__ locs1, int64_t m,
                                           const double* __restrict__ locs2, int64_t n, int64_t r0,
                                           int64_t c0, const MaternParams& mp,
-                                          const unsigned char* __restrict__ table) {
+                                          const unsigned char* table) {
   static_assert(THREADS >= 2 * kTabTile, "one thread per point");
   using L = TabLayout<F32>;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -560,7 +580,7 @@ __device__ __forceinline__ bool tab_stage(TabPoints<F32>& sm, const double* __re
   if constexpr (F32) {
     const int ex_min = q_min + 127 - sc.odd;
 #pragma unroll
-    for (int k = tid; k < TabPoints<F32>::kOct; k += THREADS) sm.oct[k] = k < ex_min ? kNone : __ldg(words + k);
+    for (int k = tid; k < TabPoints<F32>::kOct; k += THREADS) sm.oct[k] = k < ex_min ? kNone : load_word(words + k);
     if (tid < 2 * kTabTile) {
       // one FP64 fma to an integer in units of 2^{es-35}
       const double scale = __hiloint2double((1023 + sc.h - es + 35) << 20, 0);
@@ -580,7 +600,7 @@ __device__ __forceinline__ bool tab_stage(TabPoints<F32>& sm, const double* __re
   } else {
     if (tid < TabPoints<F32>::kOct) {
       const int q = 1 - tid + 2 * es + sc.odd;  // tid leading zeros
-      sm.oct[tid] = tid == 0 || tid >= 32 || q < q_min ? kNone : __ldg(words + min(max(q + 64, 0), L::kWords - 1));
+      sm.oct[tid] = tid == 0 || tid >= 32 || q < q_min ? kNone : load_word(words + min(max(q + 64, 0), L::kWords - 1));
     }
     if (tid < 2 * kTabTile) {
       const int s = 61 - (es - sc.h);
@@ -601,7 +621,7 @@ __device__ __forceinline__ bool tab_stage(TabPoints<F32>& sm, const double* __re
 // M between the points a and b; NaN when they lie outside the table.  FP64: about
 // 95 instructions, 16 of them wide products of 8 cycles a warp and scheduler; with
 // the FP64 pipe's distance n = 20,000 took 1,616 us, now 1,054 (bytes: 480).
-__device__ __forceinline__ double tab_entry(const unsigned char* __restrict__ table, const int* s_oct,
+__device__ __forceinline__ double tab_entry(const unsigned char* table, const int* s_oct,
                                             const int4& p, const int4& q) {
   const int dx = q.x - p.x, lx = q.y - p.y, dy = q.z - p.z, ly = q.w - p.w;
   const long long mid = mad_wide(2, mad_hi(ly, ly, mad_hi(lx, lx, 0)), mad_wide(dy, ly, mad_wide(dx, lx, 0LL)));
@@ -613,7 +633,7 @@ __device__ __forceinline__ double tab_entry(const unsigned char* __restrict__ ta
   const unsigned w = (unsigned)s_oct[lz];
   using L = TabLayout64;
   const uint4* const rec = reinterpret_cast<const uint4*>(table) + ((int)__funnelshift_r(h, 0u, w) + ((int)w >> 5));
-  const uint4 a = __ldg(rec), b = __ldg(rec + (L::kBins + L::kExtra));
+  const uint4 a = load_record(rec), b = load_record(rec + (L::kBins + L::kExtra));
   const unsigned u32 = __funnelshift_r(~l, ~h, w);
   const unsigned long long u = (((unsigned long long)u32 << 32) | __funnelshift_r(0u, ~l, w)) >> 1;
   unsigned A = (b.x & ((1u << kLow5) - 1u)) + __umulhi(a.z & ((1u << kLow6) - 1u), u32);
@@ -639,7 +659,7 @@ __device__ __forceinline__ double tab_entry(const unsigned char* __restrict__ ta
 // scheme it was 125, 60 of them on the integer pipe: n = 40,000 took 3.60 ms,
 // now 1.67).  The record loads bound it: a warp's 32 distances touch about
 // nine cache lines.  A matrix's rms error is 2.6e-8, against 2.5e-8 of rounding alone.
-__device__ __forceinline__ float tab_entry(const unsigned char* __restrict__ table, const int* s_oct,
+__device__ __forceinline__ float tab_entry(const unsigned char* table, const int* s_oct,
                                            const float4& a, const float4& b) {
   const float dx = b.x - a.x, lx = b.y - a.y, dy = b.z - a.z, ly = b.w - a.w;
   const float h = fmaf(dx, dx, dy * dy);                                           // exact
@@ -648,7 +668,7 @@ __device__ __forceinline__ float tab_entry(const unsigned char* __restrict__ tab
   const unsigned tb = __float_as_uint(t);
   const unsigned w = (unsigned)s_oct[(tb >> 23) & 255u];
   const unsigned lead = __funnelshift_r(tb, 0u, w);                                // tb >> (w & 31)
-  const float4 c = __ldg(reinterpret_cast<const float4*>(table) + ((int)lead + ((int)w >> 5)));
+  const float4 c = load_record(reinterpret_cast<const float4*>(table) + ((int)lead + ((int)w >> 5)));
   const float u = (t - __uint_as_float(__funnelshift_l(0u, lead, w))) + lo;        // from the left end
   return fmaf(fmaf(fmaf(c.w, u, c.z), u, c.y), u, c.x);
 }
@@ -745,7 +765,7 @@ __device__ __forceinline__ OutT tab_direct(const double* __restrict__ locs1, int
 // takes columns part * width .. + width - 1 only (width 16 or 64), where whole
 // tiles would leave SMs without a block.
 template <bool F32, typename OutT, bool kSym, int WARPS>
-__device__ __forceinline__ void tab_tile(TabTileSmem<F32, OutT>& sm, const unsigned char* __restrict__ table,
+__device__ __forceinline__ void tab_tile(TabTileSmem<F32, OutT>& sm, const unsigned char* table,
                                          const double* __restrict__ locs1, int64_t m,
                                          const double* __restrict__ locs2, int64_t n, int64_t I,
                                          int64_t J, const MaternParams& mp, OutT* __restrict__ out,
