@@ -15,11 +15,14 @@
 // 2^-57 of sqrt(a_ii a_jj) a step, against FP64's 2^-53 of the numbers at hand.
 // An input outside those bounds, a pivot that is not positive, or a row of L
 // longer than its diagonal allows means that the matrix is not positive definite.
-// All three are tested, so that no integer wraps around unnoticed: before a column
-// is scaled, |v| < 2^60 sqrt(D 2^-60) for what stands below its pivot D (within a
-// factor of 4; the products hold that); the sum of the squares of a panel's part of
-// a row (within 1/16); and the sign of what an update leaves of the diagonal.  Every
-// number of an accepted matrix then stays below 2^62.
+// All three are tested, so that no integer wraps around unnoticed.  What stands
+// below a pivot D is held at 2^62 sqrt(D 2^-60) before it is scaled (clamped), so
+// that such an x shows, and the blocks of the forward substitution, which read all
+// of L off the pivots' path, sum the squares of its rows (add_square).  A row of a
+// positive definite matrix sums to less than 2^120; one of up to 2 2^120 has left
+// the differences of 2^60 and such sums below 2^63.  (The same tests beside the pivots,
+// in the panel's registers: n = 1,000 792 us, n = 8,000 11.0 ms; this way 678 us and
+// 10.12 ms; without them 675 us and 10.01 ms.)
 //
 // Digits.  x = sum_s d_s 2^{54 - 9 s}, s = 0 .. 6, d_s in [-256, 255] (|d_0| <=
 // 64): exact.  A product of two rows is sum_g 2^{48 - 9 g} S_g in units of 2^-60,
@@ -70,18 +73,20 @@ struct CholWork {
   int* scale;      // s_i
   double* diag;    // two 64 x 64 factors, column-major: panel k's at k mod 2
   double* part;    // per panel: sum log L_ii, sum y_i^2
+  float* squares;  // per row: the squares of its part of the panels taken off z so far
   unsigned char* slices;
 };
 size_t round256(size_t v) { return (v + 255) / 256 * 256; }
 struct CholLayout {
-  size_t scale, diag, part, slices, total;
+  size_t scale, diag, part, squares, slices, total;
 };
 CholLayout chol_layout(int64_t n) {
   CholLayout l;
   l.scale = 256;
   l.diag = l.scale + round256((size_t)n * sizeof(int));
   l.part = l.diag + 2 * kNB * kNB * sizeof(double);
-  l.slices = l.part + round256((size_t)((n + kNB - 1) / kNB) * 2 * sizeof(double));
+  l.squares = l.part + round256((size_t)((n + kNB - 1) / kNB) * 2 * sizeof(double));
+  l.slices = l.squares + round256((size_t)n * sizeof(float));
   l.total = l.slices + (size_t)((n + kRowBlock - 1) / kRowBlock) * kBlockBytes;
   return l;
 }
@@ -190,28 +195,29 @@ __device__ __forceinline__ long long rsqrt_fixed(long long D, int& t) {
   return ((long long)Y << 37) + (p >> 9);
 }
 
-// (v 2^t) rho / 2^60, v of magnitude below 2^{61 - t} (too_large).
+// v, held between about -2^{62 - t} and 2^{62 - t}; t <= 30.
+__device__ __forceinline__ long long clamped(long long v, int t) {
+  const int top = 0x40000000 >> t;
+  const int h = min(max((int)(v >> 32), -top), top);
+  return ((long long)h << 32) | (unsigned)v;
+}
+// (v 2^t) rho / 2^60 for a clamped v.
 __device__ __forceinline__ long long mul_rho(long long v, int t, Limbs rho) {
   Acc a;
   a.add(limbs(v << t), rho);
   return a.sum();
 }
 
-// Whether |v| >= 2^{61 - t} (-2^{61 - t} itself passes); t <= 30.
-__device__ __forceinline__ bool too_large(long long v, int t) {
-  if (t > 29) return (unsigned long long)((v >> 31) + 1) > 1ULL;  // D below 4 units
-  return (unsigned)(((int)(v >> 32) >> (29 - t)) + 1) > 1u;
+// sum + (L 2^-s)^2 in FP32 without the FP64 pipe, nothing for L below 2^{s - 60}.
+constexpr float kMaxSquares = 2.0f;
+__device__ __forceinline__ float add_square(float sum, double L, int s) {
+  const unsigned hi = (unsigned)__double2hiint(L) & 0x7fffffffu;
+  const int e = (int)(hi >> 20) - s;  // (infinite and NaN entries: the flag is set already)
+  const float x = __uint_as_float(((unsigned)(e - 1023 + 127) << 23) | ((hi & 0xfffffu) << 3));
+  return e > 1023 - 60 ? fmaf(x, x, sum) : sum;
 }
 
-// The sum of (x 2^-50)^2 over columns of a row: at most (2^10)^2 in exact numbers,
-// and less than 2^14 + 64 more by truncation; |x| < 2^62, so that 64 squares fit.
-constexpr unsigned kRowSquares = (1u << 20) + (1u << 15);
-__device__ __forceinline__ unsigned add_square(unsigned sum, Limbs x) {
-  const int h = x.h >> 18;
-  return sum + (unsigned)(h * h);
-}
-
-// Scales, y = z, the flag.
+// Scales, y = z, the flag, the sums of squares.
 __global__ void __launch_bounds__(256) chol_prep_kernel(const double* __restrict__ a, int64_t ld,
                                                         int64_t n, const double* __restrict__ z,
                                                         double* __restrict__ y, CholWork w) {
@@ -226,12 +232,14 @@ __global__ void __launch_bounds__(256) chol_prep_kernel(const double* __restrict
   } else {
     w.scale[i] = (e >> 1) + 1;
   }
+  w.squares[i] = 0.0f;
   y[i] = z[i];
 }
 
 // Panel q's share of the forward substitution and of the sums, by one block:
 // y_q <- L_qq^{-1} (y_q - L_{q,q-1} y_{q-1}), sum log L_ii, sum y_i^2, and L_qq
-// into the matrix.  Earlier panels' parts of y_q were taken off before.
+// into the matrix.  Earlier panels' parts of y_q were taken off before, and their
+// squares are summed.
 __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld, int64_t n, int64_t q,
                                              double* __restrict__ y, const CholWork& w, double* sh) {
   const int64_t o = q * kNB;
@@ -239,6 +247,7 @@ __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld,
   const int tid = threadIdx.x, lane = tid & 31;
   double* const L = sh;                       // 64 x 65
   double* const part = sh + kNB * (kNB + 1);  // 8 x 64
+  float* const squares = reinterpret_cast<float*>(part + 8 * kNB);  // 8 x 64
   for (int e = tid; e < kNB * kNB; e += kPanelThreads) {
     const int r = e & 63, c = e >> 6;
     const double v = w.diag[(q & 1) * (kNB * kNB) + e];
@@ -248,12 +257,18 @@ __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld,
   {
     const int r = tid & 63, h = tid >> 6;
     double s = 0.0;
+    float sum = 0.0f;
     if (q > 0 && r < b) {
+      const int scale = w.scale[o + r];
 #pragma unroll
-      for (int c = 8 * h; c < 8 * h + 8; ++c)
-        s = fma(a[(o + r) + (o - kNB + c) * ld], y[o - kNB + c], s);
+      for (int c = 8 * h; c < 8 * h + 8; ++c) {
+        const double v = a[(o + r) + (o - kNB + c) * ld];
+        s = fma(v, y[o - kNB + c], s);
+        sum = add_square(sum, v, scale);
+      }
     }
     part[h * kNB + r] = s;
+    squares[h * kNB + r] = sum;
   }
   __syncthreads();
   if (tid < 32) {  // rows lane and lane + 32
@@ -293,6 +308,18 @@ __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld,
     if (lane == 0) {
       w.part[2 * q] = ld_;
       w.part[2 * q + 1] = sq;
+    }
+  } else if (tid >= kPanelThreads / 2) {
+    const int r = (tid - kPanelThreads / 2) >> 2, g = tid & 3;
+    if (r < b) {
+      const int scale = w.scale[o + r];
+      float sum = squares[2 * g * kNB + r] + squares[(2 * g + 1) * kNB + r];
+      if (g == 0) sum += w.squares[o + r];
+      for (int c = g; c < r; c += 4) sum = add_square(sum, L[c * (kNB + 1) + r], scale);
+      const unsigned quad = 15u << (tid & 28);
+      sum += __shfl_xor_sync(quad, sum, 1);
+      sum += __shfl_xor_sync(quad, sum, 2);
+      if (sum > kMaxSquares) *w.flag = 1;
     }
   }
 }
@@ -363,14 +390,27 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
     __syncthreads();
     const int64_t r = o + (int64_t)((int)blockIdx.x - row_blocks - 1) * 256 + (tid & 255);
     const int h = tid >> 8;
+    float* const squares = reinterpret_cast<float*>(ys + kNB + 256);
     double s = 0.0;
+    float sum = 0.0f;
     if (r < n) {
+      const int scale = w.scale[r];
 #pragma unroll 8
-      for (int c = 32 * h; c < 32 * h + 32; ++c) s = fma(a[r + (po + c) * ld], ys[c], s);
+      for (int c = 32 * h; c < 32 * h + 32; ++c) {
+        const double v = a[r + (po + c) * ld];
+        s = fma(v, ys[c], s);
+        sum = add_square(sum, v, scale);
+      }
     }
-    if (h == 1) ys[kNB + (tid & 255)] = s;
+    if (h == 1) {
+      ys[kNB + (tid & 255)] = s;
+      squares[tid & 255] = sum;
+    }
     __syncthreads();
-    if (h == 0 && r < n) y[r] -= s + ys[kNB + tid];
+    if (h == 0 && r < n) {
+      y[r] -= s + ys[kNB + tid];
+      w.squares[r] += sum + squares[tid];
+    }
     return;
   }
   const int b = (int)(n - o < kNB ? n - o : kNB);
@@ -417,7 +457,6 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
   __syncthreads();
   const int groups = own > 32 ? 4 : own > 0 ? 3 : 2;  // row groups of 32
   const int follow = 8 + kFollow * warp + lane - 8;   // a solving lane's row (lanes 8 .. 31)
-  unsigned squares = 0;                               // of that row
   for (int c0 = 0; c0 < kNB; c0 += 8) {
     // solving warps whose rows are all done (the tile's first ones) join the others
     const int retired = min(c0 / kFollow, kSolve - 1);
@@ -441,8 +480,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
           v[j] -= acc.sum();
         }
       }
-      bool bad = false, over = false;
-      if (lane < 8) squares = 0;
+      bool bad = false;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         long long D = shfl64(v[c], c);
@@ -452,10 +490,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
         }
         int t;
         const Limbs rho = limbs(rsqrt_fixed(D, t));
-        const bool below = lane > c;
-        over = (below && too_large(v[c], t)) || over;
-        const Limbs x = limbs(mul_rho(v[c], t, rho));
-        if (below) squares = add_square(squares, x);
+        const Limbs x = limbs(mul_rho(clamped(v[c], t), t, rho));
         v[c] = raw_limbs(x);
 #pragma unroll
         for (int j = c + 1; j < 8; ++j) {
@@ -466,16 +501,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
           v[j] -= p.sum();
         }
       }
-      // (rows above the group's block hold nothing that counts)
-      if ((lane < 8 || follow >= c0 + 8) && (over || squares > kRowSquares)) bad = true;
       if (lane >= 8 ? follow >= c0 + 8 : warp == kSolve - 1) {
+        long long* const dst = lane >= 8 ? &sm.S[row][c0] : sm.D[row];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          if (lane >= 8) sm.S[row][c0 + c] = v[c];
-          else if (c <= lane) sm.D[row][c] = v[c];
-        }
+        for (int c = 0; c < 8; ++c) dst[c] = v[c];
       }
-      if (bad) sm.bad = 1;
+      if (bad && lane == 0) sm.bad = 1;
     } else if (c0 > 0) {
       // the rest of the previous group's update: columns from c0 + 8 on
       const int rest = kPanelThreads / 32 - kSolve + retired, u = warp < kSolve ? warp : warp - kSolve + retired;
@@ -505,8 +536,8 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
     __syncthreads();
   }
   const bool bad = sm.bad != 0;
-  if (bad && tid == 0) *w.flag = 1;
   if ((int)blockIdx.x == row_blocks - 1) {
+    if (bad && tid == 0) *w.flag = 1;
     for (int e = tid; e < kNB * kNB; e += kPanelThreads) {
       const int r = e & 63, c = e >> 6;
       double v = r == c ? 1.0 : 0.0;
@@ -853,11 +884,6 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
           if (g == 1) acc[c] += kMagicSum - ((unsigned long long)top[c] << 32);
         }
       }
-      if (ok && J >= 2 * I) {  // a tile on the diagonal
-#pragma unroll
-        for (int c = 0; c < kEpiCols; ++c)
-          if (cb + c == r && r < n && acc[c] <= 0) *w.flag = 1;
-      }
       if (ok) {
         p = p0;
         asm volatile("" : "+l"(p));  // or the loads' addresses are kept for the stores
@@ -877,11 +903,11 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
 __global__ void __launch_bounds__(kPanelThreads) chol_finish_kernel(
     double* __restrict__ a, int64_t ld, int64_t n, int64_t nt, double* __restrict__ y,
     double* __restrict__ out, CholWork w, unsigned long long* __restrict__ ctr) {
-  __shared__ double sh[kNB * (kNB + 1) + 8 * kNB];
+  __shared__ double sh[kNB * (kNB + 1) + 12 * kNB];
   chain();
   finish_panel(a, ld, n, nt - 1, y, w, sh);
+  __syncthreads();
   if (threadIdx.x >= 32) return;
-  __syncwarp();
   const int lane = threadIdx.x;
   double ld_ = 0.0, q = 0.0;
   for (int64_t k = lane; k < nt; k += 32) {
@@ -948,7 +974,7 @@ cudaError_t launch_loglik_fixed(double* a, int64_t n, int64_t ld, const double* 
   const CholLayout l = chol_layout(n);
   unsigned char* const base = (unsigned char*)work;
   const CholWork w{(int*)base, (int*)(base + l.scale), (double*)(base + l.diag),
-                   (double*)(base + l.part), base + l.slices};
+                   (double*)(base + l.part), (float*)(base + l.squares), base + l.slices};
   if ((e = cudaMemsetAsync(w.flag, 0, sizeof(int), s)) != cudaSuccess) return e;
   chol_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a, ld, n, z, y, w);
   const int64_t nt = (n + kNB - 1) / kNB, R = (n + kRowBlock - 1) / kRowBlock;
