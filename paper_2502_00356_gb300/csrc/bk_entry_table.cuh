@@ -810,7 +810,9 @@ __device__ __forceinline__ void tab_tile(TabTileSmem<F32, OutT>& sm, const unsig
       OutT* const po = p0 + 32 * (k & 1) + (c - cw) * ld;
       if (r0 + i >= m) continue;
       if (use_table) {
-        const OutT v = *po;
+        OutT v;
+        if constexpr (kSym) v = sm.tile[i][c];  // (the matrix may be host memory)
+        else v = *po;
         if (v == v) continue;
       }
       const OutT v = tab_direct<F32, OutT>(locs1, m, r0 + i, locs2, n, c0 + c, mp);
