@@ -135,7 +135,7 @@ bk_status check_work(const void* d_work) {
 }  // namespace
 
 size_t matern_scratch_bytes(bool table) {
-  return kEntryTableOffset + (table ? std::max(entry_table_bytes(false), entry_table_bytes(true)) : 0);
+  return table ? std::max(entry_table_bytes(false), entry_table_bytes(true)) : kDecayTableBytes;
 }
 
 void* matern_scratch(bk_opts& o, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
@@ -143,8 +143,8 @@ void* matern_scratch(bk_opts& o, int64_t rows, int64_t cols, double sigma2, doub
   if (d_work == nullptr) return nullptr;
   if (entry_table_pays(rows, cols) && work_bytes >= matern_scratch_bytes(true) &&
       entry_table_applies(o, sigma2, beta, nu))
-    return (char*)d_work + kEntryTableOffset;
-  if (o.compute == BK_F64 && o.d_cosh_table == nullptr && work_bytes >= kEntryTableOffset)
+    return d_work;
+  if (o.compute == BK_F64 && o.d_cosh_table == nullptr && work_bytes >= kDecayTableBytes)
     o.d_cosh_table = (double*)d_work;
   return nullptr;
 }

@@ -83,10 +83,14 @@ __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
   __shared__ TabBuildSmem sm;
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
   const BatchInstance& b = inst[blockIdx.y];
-  if (!b.table) return;
+  if (!b.table) {
+    if (!F32 && blockIdx.x == 0 && threadIdx.x == 0)
+      *reinterpret_cast<double*>(tables + (size_t)blockIdx.y * TabLayout<F32>::kStride) = -1.0;
+    return;
+  }
   const MaternParams mp = b.mp;
   tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, b.n <= kTabScan, b.locs, b.n, b.locs, b.n,
-                       tables + (size_t)blockIdx.y * TabLayout<F32>::kBytes);
+                       tables + (size_t)blockIdx.y * TabLayout<F32>::kStride + TabLayout<F32>::kFront);
 }
 
 // Persistent kernel as matern_batched_kernel, in tiles of 64.
@@ -121,7 +125,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
       }
       int64_t I, J;
       tri_tile(w - __ldg(prefix + k), I, J);
-      tab_tile<F32, OutT, true, WARPS>(sm, tables + (size_t)k * TabLayout<F32>::kBytes,
+      tab_tile<F32, OutT, true, WARPS>(sm, tables + (size_t)k * TabLayout<F32>::kStride + TabLayout<F32>::kFront,
                                        cur.locs, cur.n, cur.locs, cur.n, I, J, cur.mp, (OutT*)cur.out, cur.ld, 0, kTabTile,
                                        cur.table != 0);
     }
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
 
 }  // namespace
 
-size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kBytes : TabLayout64::kBytes; }
+size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kStride : TabLayout64::kStride; }
 
 // entry_table_size (the header): from 2^19 entries on (n = 725) a matrix is worth
 // a table, which costs about 15 us: n = 777 takes 29 us with it, 63 without; at
@@ -187,8 +191,8 @@ cudaError_t launch_matern_sym_table(const double* locs, int64_t n, double sigma2
                                     bk_dtype compute, void* table, cudaStream_t s,
                                     const SymRange& range) {
   const MaternParams mp = matern_params_host(sigma2, beta, nu);
-  unsigned char* const tab = (unsigned char*)table;
   const bool f32 = compute == BK_F32 && out_t == BK_F32;
+  unsigned char* const tab = (unsigned char*)table + (f32 ? TabLayout32::kFront : TabLayout64::kFront);
   if (range.fill_table) {
     const cudaError_t e = f32 ? build_table<true>(mp, locs, n, locs, n, tab, s)
                               : build_table<false>(mp, locs, n, locs, n, tab, s);
@@ -219,8 +223,8 @@ cudaError_t launch_matern_block_table(const double* locs1, int64_t m, const doub
                                       double sigma2, double beta, double nu, void* out, int64_t ld,
                                       bk_dtype out_t, bk_dtype compute, void* table, cudaStream_t s) {
   const MaternParams mp = matern_params_host(sigma2, beta, nu);
-  unsigned char* const tab = (unsigned char*)table;
   const bool f32 = compute == BK_F32 && out_t == BK_F32;
+  unsigned char* const tab = (unsigned char*)table + (f32 ? TabLayout32::kFront : TabLayout64::kFront);
   const cudaError_t e = f32 ? build_table<true>(mp, locs1, m, locs2, n, tab, s)
                             : build_table<false>(mp, locs1, m, locs2, n, tab, s);
   if (e != cudaSuccess) return e;

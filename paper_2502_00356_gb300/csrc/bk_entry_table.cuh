@@ -74,6 +74,12 @@ struct TabLayout {
   static constexpr int kNaN = kBins, kZero = kBins + 2, kExtra = 3;
   static constexpr int kWords = F32 ? 256 : 128;
   static constexpr size_t kBytes = (size_t)(kBins + kExtra) * kRecord + kWords * sizeof(int);
+  // In front of an FP64 table, for the entries beyond it: the plain form's
+  // e^{-2 nu h} on kCoshTab's steps (n = 4,001, beta = 0.002, most entries between
+  // x = 90 and 700: 980 us without it, 920 with; the per-entry writer 810).  Its
+  // first entry is negative when it was not filled.
+  static constexpr size_t kFront = F32 ? 0 : (size_t)kCoshTabSize * sizeof(double);
+  static constexpr size_t kStride = (kFront + kBytes + 255) / 256 * 256;
 };
 using TabLayout64 = TabLayout<false>;
 using TabLayout32 = TabLayout<true>;
@@ -405,7 +411,16 @@ __device__ __forceinline__ void tab_build_block(TabBuildSmem& sm, const MaternPa
           tab_octave<F32>((int)threadIdx.x, mp);
   }
   // the intervals of binades up to r2_max's
-  const int o_max = min((int)((unsigned)__double2hiint(r2_max) >> 20) - (int)e0, kTabOct - 1);
+  const int o_top = (int)((unsigned)__double2hiint(r2_max) >> 20) - (int)e0, o_max = min(o_top, kTabOct - 1);
+  if constexpr (!F32) {
+    double* const front = reinterpret_cast<double*>(table - L::kFront);
+    if (o_top >= kTabOct) {  // distances beyond the table
+      for (int i = block + blocks * (int)threadIdx.x; i < kCoshTabSize; i += blocks * kTabThreads)
+        front[i] = decay_entry(mp.nu, i, kExp2Tab);
+    } else if (block == 0 && threadIdx.x == 0) {
+      front[0] = -1.0;
+    }
+  }
   int bins = 0;
 #pragma unroll
   for (int o = 0; o < kTabOct; ++o)
@@ -684,11 +699,16 @@ struct NanSeen {
 
 // The direct evaluation of one entry, for pairs outside the table; out of
 // line, so that the common path keeps its registers.
-static __device__ __noinline__ double matern_direct64(const Loc& a, const Loc& b,
-                                                      const MaternParams& mp) {
+static __device__ __noinline__ double matern_direct64(double px, double py, double qx, double qy,
+                                                      const MaternParams& mp, const double* decay) {
   Tally tl{0u, 0u, 0u, 0u, 0u, 0u, 0u};
   unsigned evals = 0;
-  const FormF64 f{kExp2Tab, false, 0.0};
+  const FormF64 f{kExp2Tab, false, 0.0, decay};
+  Loc a, b;
+  a.x = px;
+  a.y = py;
+  b.x = qx;
+  b.y = qy;
   return f.matern(a, b, mp, tl, evals);
 }
 static __device__ __noinline__ float matern_direct32(const Loc& a, const Loc& b,
@@ -736,24 +756,30 @@ __device__ __forceinline__ void tab_transpose(const OutT (*tile)[kTabTile + 1], 
   }
 }
 
-// One entry by the direct evaluation.
+// log M at most, for x >= 1: log c + (nu - 1/2) log x - x + (4 nu^2 - 1)/(8 x) + 0.23.
+__device__ __forceinline__ float tab_log_bound(float x, const MaternParams& mp) {
+  return fmaf(fmaxf(f32_trunc(mp.nu) - 0.5f, 0.0f), __logf(x), f32_trunc(mp.log_pref)) - x + 1.5f;
+}
+
+// One entry by the direct evaluation, 0 where it underflows (below 2^-1080, 2^-152).
 template <bool F32, typename OutT>
 __device__ __forceinline__ OutT tab_direct(const double* __restrict__ locs1, int64_t m, int64_t i,
                                            const double* __restrict__ locs2, int64_t n, int64_t j,
-                                           const MaternParams& mp) {
-  Loc p, q;
-  p.x = locs1[i];
-  p.y = locs1[m + i];
-  q.x = locs2[j];
-  q.y = locs2[n + j];
+                                           const MaternParams& mp, const double* decay) {
+  const double px = locs1[i], py = locs1[m + i], qx = locs2[j], qy = locs2[n + j];
+  const double wx = qx - px, wy = qy - py;
+  if (wx == 0.0 && wy == 0.0) return (OutT)mp.sigma2;  // the diagonal, without a call
+  const float dx = f32_trunc(wx), dy = f32_trunc(wy), x = sqrtf(fmaf(dx, dx, dy * dy)) * mp.inv_beta_f;
+  if (x > 64.0f && x < 1e6f && tab_log_bound(x, mp) < (sizeof(OutT) == 4 ? -106.0f : -749.0f)) return (OutT)0;
   if constexpr (F32) {
-    split_f(p.x, p.xh, p.xl);
-    split_f(p.y, p.yh, p.yl);
-    split_f(q.x, q.xh, q.xl);
-    split_f(q.y, q.yh, q.yl);
+    Loc p, q;
+    split_f(px, p.xh, p.xl);
+    split_f(py, p.yh, p.yl);
+    split_f(qx, q.xh, q.xl);
+    split_f(qy, q.yh, q.yl);
     return matern_direct32(p, q, mp);
   } else {
-    return to_out<OutT>(matern_direct64(p, q, mp));
+    return to_out<OutT>(matern_direct64(px, py, qx, qy, mp, *decay > 0.0 ? decay : nullptr));
   }
 }
 
@@ -815,7 +841,8 @@ __device__ __forceinline__ void tab_tile(TabTileSmem<F32, OutT>& sm, const unsig
         else v = *po;
         if (v == v) continue;
       }
-      const OutT v = tab_direct<F32, OutT>(locs1, m, r0 + i, locs2, n, c0 + c, mp);
+      const OutT v = tab_direct<F32, OutT>(locs1, m, r0 + i, locs2, n, c0 + c, mp,
+                                           reinterpret_cast<const double*>(table - TabLayout<F32>::kFront));
       *po = v;
       if constexpr (kSym) sm.tile[i][c] = v;
     }

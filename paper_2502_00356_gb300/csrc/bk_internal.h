@@ -83,11 +83,11 @@ cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* desc
                                  cudaStream_t s);
 int batched_table_max_ctas(bool f32, bk_dtype out_t, int warps);
 
-// The scratch of one Matern call: the plain form's e^{-2 nu h} table, and behind
-// it the entry table when the matrix is worth one.  matern_scratch returns the
-// place of the entry table when the call takes it, else null, with
-// o.d_cosh_table set to the scratch when it fits and the caller gave none.
-constexpr size_t kEntryTableOffset = (size_t)BK_COSH_TABLE_LEN * sizeof(double);
+// The scratch of one Matern call: the plain form's e^{-2 nu h} table, or the entry
+// table when the matrix is worth one.  matern_scratch returns the place of the entry
+// table when the call takes it, else null, with o.d_cosh_table set to the scratch
+// when it fits and the caller gave none.
+constexpr size_t kDecayTableBytes = (size_t)BK_COSH_TABLE_LEN * sizeof(double);
 size_t matern_scratch_bytes(bool table);
 void* matern_scratch(bk_opts& o, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
                      void* d_work, size_t work_bytes);

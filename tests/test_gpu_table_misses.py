@@ -1,0 +1,60 @@
+"""Entries that an entry table does not hold: far pairs (evaluated with the plain
+form's e^{-2 nu h}, or zero where they underflow), coincident ones, values at
+the lower end of FP32."""
+import pytest
+
+import paper_2502_00356_gb300 as bk
+from paper_2502_00356_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    bk.build()
+    return torch.device("cuda:0")
+
+
+def grid(n, seed, dev, scale=1.0):
+    return torch.as_tensor(inputs.morton_sorted(inputs.jittered_grid(n, seed=seed)) * scale, device=dev)
+
+
+def direct(**kw):
+    """Options that ask for the per-entry evaluation."""
+    return bk.make_opts(counters=torch.zeros(bk.BK_NUM_COUNTERS, dtype=torch.int64, device="cuda"), **kw)
+
+
+@pytest.mark.parametrize("nu", [0.02, 0.5, 2.3, 10.0])
+@pytest.mark.parametrize("width", [150.0, 700.0, 2000.0, 40000.0])
+@pytest.mark.parametrize("block", [False, True])
+def test_far_pairs(dev, nu, width, block):
+    """x up to `width` and beyond: the tables end at 90, FP64 underflows past 745,
+    FP32 past 104.  Twice the direct forms' bounds (1e-13, 1e-6), and an ulp of
+    the smallest numbers."""
+    n = 760
+    L, M = grid(n, 1, dev, width), grid(900, 2, dev, width)
+    for dtype, compute in ((torch.float64, bk.BK_F64), (torch.float32, bk.BK_F64), (torch.float32, bk.BK_F32)):
+        call = (lambda o: bk.bk_matern_tile2(L, M, 1.5, 1.0, nu, dtype=dtype, opts=o)) if block else \
+               (lambda o: bk.bk_matern_tile(L, 1.5, 1.0, nu, dtype=dtype, opts=o))
+        got, want = call(bk.make_opts(compute=compute)).double(), call(direct(compute=compute)).double()
+        torch.cuda.synchronize()
+        small = 1e-300 if dtype == torch.float64 else 2e-38
+        tol = 4e-13 if dtype == torch.float64 else 2e-6 if compute == bk.BK_F32 else 2.0 ** -23
+        assert bool(((got - want).abs() <= tol * want.abs() + small).all())
+        assert bool((got >= 0).all())
+
+
+def test_every_path_to_an_entry_in_one_matrix(dev):
+    """Coincident, near, tabulated, far and underflowing pairs side by side, more
+    points than the scan of the distances takes (8,192): the table is complete."""
+    n = 9000
+    L = torch.cat([grid(4000, 3, dev, 1.0), grid(3000, 4, dev, 1e-3) + 5.0, grid(2000, 5, dev, 3000.0)], dim=1)
+    L[:, 8990:] = L[:, :10]
+    L = L.contiguous()
+    got, want = (bk.bk_matern_tile(L, 0.7, 1.0, 1.2, opts=o) for o in (None, direct()))
+    torch.cuda.synchronize()
+    assert bool(((got - want).abs() <= 4e-13 * want.abs() + 1e-300).all())
+    assert bool((got.diagonal() == 0.7).all()) and float(got[0, 8990]) == 0.7
