@@ -685,7 +685,11 @@ __device__ __forceinline__ float tab_entry(const unsigned char* table, const int
   const unsigned lead = __funnelshift_r(tb, 0u, w);                                // tb >> (w & 31)
   const float4 c = load_record(reinterpret_cast<const float4*>(table) + ((int)lead + ((int)w >> 5)));
   const float u = (t - __uint_as_float(__funnelshift_l(0u, lead, w))) + lo;        // from the left end
-  return fmaf(fmaf(fmaf(c.w, u, c.z), u, c.y), u, c.x);
+  // at least 0: where a record's coefficients are subnormal numbers the cubic may
+  // end a few of their units below (a NaN stays)
+  float v;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(v) : "f"(fmaf(fmaf(fmaf(c.w, u, c.z), u, c.y), u, c.x)));
+  return v;
 }
 
 // Keeps a NaN among the values it has seen.

@@ -58,3 +58,18 @@ def test_every_path_to_an_entry_in_one_matrix(dev):
     torch.cuda.synchronize()
     assert bool(((got - want).abs() <= 4e-13 * want.abs() + 1e-300).all())
     assert bool((got.diagonal() == 0.7).all()) and float(got[0, 8990]) == 0.7
+
+
+@pytest.mark.parametrize("sigma2,width", [(1e-20, 62.0), (1e-20, 70.0), (1e-10, 75.0), (1.0, 100.0), (1e-20, 45.0)])
+def test_no_fp32_entry_is_negative(dev, sigma2, width):
+    """Down to where FP32 ends (2^-149) a covariance is never below zero, and the
+    subnormal ones are within a few of their units of the FP64 values."""
+    L, M = grid(2500, 6, dev, width), grid(1700, 7, dev, width)
+    for nu in (0.3, 1.5, 7.0):
+        for got, want in ((bk.bk_matern_tile(L, sigma2, 1.0, nu, dtype=torch.float32), bk.bk_matern_tile(L, sigma2, 1.0, nu)),
+                          (bk.bk_matern_tile2(L, M, sigma2, 1.0, nu, dtype=torch.float32),
+                           bk.bk_matern_tile2(L, M, sigma2, 1.0, nu))):
+            torch.cuda.synchronize()
+            assert bool((got >= 0).all()), float(got.min())
+            low = want < 2.0 ** -130
+            assert bool(low.any()) and float((got.double() - want)[low].abs().max()) <= 2.0 ** -130 * 2e-6 + 64 * 2.0 ** -149
