@@ -136,10 +136,15 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
 
 size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kStride : TabLayout64::kStride; }
 
-// entry_table_size (the header): from 2^19 entries on (n = 725) a matrix is worth
-// a table, which costs about 15 us: n = 777 takes 29 us with it, 63 without; at
-// half the entries both take about 25, and such matrices keep the direct path,
-// whose results do not depend on whether the caller has scratch memory.
+// entry_table_size (the header): a matrix is worth a table, which costs about 13 us,
+// from 2^19 entries on (n = 725) in every form, as the writers without one are bound
+// by one entry's latency there.  n = 800, beta = 0.1, nu = 0.8: 27 us with it, without
+// 66 (FP64), 44 (FP32), 34 (learned); blocks of 520,000 entries 24 with it, without
+// 80, 44, 31.  Smaller ones keep the direct path, whose results do not depend on
+// whether the caller has scratch memory.  Stored to host memory FP64 and FP32 gain too
+// (n = 800: 53 and 36 us, without 75 and 49 to 61); the learned form takes 36 (38) at
+// n = 800, 47 (42) at 900, 44 (41) at 1,024, 57 (58) at 1,280, 85 (88) at 1,450, and
+// keeps the rule, so that a matrix is the same wherever it is stored.
 bool entry_table_pays(int64_t rows, int64_t cols) { return entry_table_size(rows, cols); }
 
 bool entry_table_applies(const bk_opts& o, double sigma2, double beta, double nu) {
@@ -150,9 +155,17 @@ bool entry_table_applies(const bk_opts& o, double sigma2, double beta, double nu
 namespace {
 
 // Whole tiles where they fill the SMs' four slots once, else quarters of 16
-// columns (n = 777: 91 tiles on 152 SMs, 14.8 us whole).
-int tile_width(int64_t ntiles) {
-  return ntiles < (int64_t)current_sm_count() * 4 ? kTabTile / 4 : kTabTile;
+// columns (n = 777: 91 tiles on 152 SMs, 14.8 us whole).  Over the link to host
+// memory a part's transposed columns of 16 rows are pieces of lines, so halves there
+// (FP32: n = 850 48.5 us in quarters, 44.6 in halves; n = 1,280 61.0, 56.5), and
+// whole tiles where the matrix's columns do not start on 32 bytes, from 1.5 tiles an
+// SM on (n = 1,450 99.7 us in quarters, 87.4 in halves, 85.2 whole; n = 1,837 147.8,
+// 131.3, 123.3; FP64 218, 199, 194; but FP64 n = 2,048 199 in halves, 205 whole).
+int tile_width(int64_t ntiles, bool host, int64_t column_bytes) {
+  const int64_t sms = current_sm_count();
+  if (ntiles >= 4 * sms) return kTabTile;
+  if (!host) return kTabTile / 4;
+  return column_bytes % 32 != 0 && 2 * ntiles >= 3 * sms ? kTabTile : kTabTile / 2;
 }
 
 // Launches a kernel so that it may be scheduled while the one before it still
@@ -207,7 +220,7 @@ cudaError_t launch_matern_sym_table(const double* locs, int64_t n, double sigma2
     ntiles = (j1 * nb - j1 * (j1 - 1) / 2) - col_base;
   }
   if (ntiles > 2147483647) return cudaErrorInvalidConfiguration;
-  const int width = tile_width(ntiles);
+  const int width = tile_width(ntiles, range.host, ld * (out_t == BK_F64 ? 8 : 4));
   const unsigned grid = (unsigned)(ntiles * (kTabTile / width));
   if (f32)
     return launch_writer(matern_table_kernel<true, float, true>, grid, s, tab, locs, n, locs, n, mp,
@@ -230,7 +243,7 @@ cudaError_t launch_matern_block_table(const double* locs1, int64_t m, const doub
   if (e != cudaSuccess) return e;
   const int64_t tm = (m + kTabTile - 1) / kTabTile, tn = (n + kTabTile - 1) / kTabTile;
   if (tm * tn > 2147483647) return cudaErrorInvalidConfiguration;
-  const int width = tile_width(tm * tn);
+  const int width = tile_width(tm * tn, false, 0);
   const unsigned grid = (unsigned)(tm * tn * (kTabTile / width));
   if (f32)
     return launch_writer(matern_table_kernel<true, float, false>, grid, s, tab, locs1, m, locs2, n, mp,

@@ -792,8 +792,8 @@ __device__ __forceinline__ OutT tab_direct(const double* __restrict__ locs1, int
 // w + WARPS, ..., two rows at a time so that the loads of one entry overlap the
 // arithmetic of the other.  kSym: the transposed block (J, I) is written too.
 // use_table false: every entry by the direct evaluation.  part, width: the block
-// takes columns part * width .. + width - 1 only (width 16 or 64), where whole
-// tiles would leave SMs without a block.
+// takes columns part * width .. + width - 1 only (width 16, 32 or 64: tile_width),
+// where whole tiles would leave SMs without a block.
 template <bool F32, typename OutT, bool kSym, int WARPS>
 __device__ __forceinline__ void tab_tile(TabTileSmem<F32, OutT>& sm, const unsigned char* table,
                                          const double* __restrict__ locs1, int64_t m,

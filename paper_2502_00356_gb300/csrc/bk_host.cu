@@ -172,7 +172,11 @@ bk_status bk_matern_tile_host(const double* h_locs, int64_t n, double sigma2, do
   cudaError_t e = cudaMemcpyAsync(d_locs, h_locs, (size_t)n * 2 * sizeof(double),
                                   cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return check_cuda(e, "bk_matern_tile_host: locations to the device");
-  if (d_out != nullptr) return check_cuda(launch(d_out, ld, SymRange{}), "bk_matern_tile_host launch");
+  if (d_out != nullptr) {
+    SymRange whole;
+    whole.host = true;
+    return check_cuda(launch(d_out, ld, whole), "bk_matern_tile_host launch");
+  }
 
   // Staged: all panel kernels first (each followed by its event), then the
   // copies of each panel's columns on the copy stream.

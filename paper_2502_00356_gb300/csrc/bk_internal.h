@@ -23,10 +23,11 @@ bk_status check_cuda(cudaError_t e, const char* what);
 // written in block-column order; j1 < 0 means the whole matrix.  fill_table:
 // whether a launch refills the caller's tables (e^{-2 nu h}, or the entry
 // table; a caller writing several ranges of one matrix fills them with the
-// first).
+// first).  host: the matrix is in host memory.
 struct SymRange {
   int64_t j0 = 0, j1 = -1;
   bool fill_table = true;
+  bool host = false;
 };
 
 // ---- plain FP64 form (bk_plain.cu) ----

@@ -73,3 +73,17 @@ def test_no_fp32_entry_is_negative(dev, sigma2, width):
             assert bool((got >= 0).all()), float(got.min())
             low = want < 2.0 ** -130
             assert bool(low.any()) and float((got.double() - want)[low].abs().max()) <= 2.0 ** -130 * 2e-6 + 64 * 2.0 ** -149
+
+
+@pytest.mark.parametrize("n,pad", [(725, 0), (733, 4), (800, 0), (850, 0), (961, 7), (1343, 0), (1345, 0), (1450, 1), (1537, 7)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_a_matrix_is_the_same_in_host_memory(dev, n, pad, dtype):
+    """Halves of tiles, or whole ones (columns that do not start on 32 bytes, from
+    n = 1,345 on), where a matrix in device memory takes quarters."""
+    L = inputs.morton_sorted(inputs.jittered_grid(n, seed=8))
+    want = bk.bk_matern_tile(torch.as_tensor(L, device=dev), 0.9, 0.1, 1.3, dtype=dtype)
+    got = torch.full((n, n + pad), -1.0, dtype=dtype, pin_memory=True)
+    work = torch.empty(bk.matern_tile_host_workspace(n, dtype, staged=False), dtype=torch.uint8, device=dev)
+    bk.bk_matern_tile_host(torch.as_tensor(L).pin_memory(), 0.9, 0.1, 1.3, got, work)
+    torch.cuda.synchronize()
+    assert torch.equal(got[:, :n], want.cpu()) and bool((got[:, n:] == -1.0).all())
