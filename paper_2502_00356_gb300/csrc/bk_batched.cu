@@ -349,7 +349,7 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
       (size_t)count * entry_table_bytes(o.compute == BK_F32 && dtype == BK_F32);
   void *d_inst = nullptr, *d_tables = nullptr;
   if (pays && count <= 65535 && table_bytes <= ((size_t)1 << 30) &&
-      entry_table_applies(o, 1.0, 1.0, 1.0)) {
+      entry_table_applies(o, dtype, 1.0, 1.0, 1.0)) {
     if (cudaMalloc(&d_inst, (size_t)count * batched_instance_bytes()) != cudaSuccess ||
         cudaMalloc(&d_tables, table_bytes) != cudaSuccess) {
       (void)cudaGetLastError();  // without them the kernel evaluates every entry itself

@@ -138,11 +138,11 @@ size_t matern_scratch_bytes(bool table) {
   return table ? std::max(entry_table_bytes(false), entry_table_bytes(true)) : kDecayTableBytes;
 }
 
-void* matern_scratch(bk_opts& o, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
+void* matern_scratch(bk_opts& o, bk_dtype out_t, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
                      void* d_work, size_t work_bytes) {
   if (d_work == nullptr) return nullptr;
   if (entry_table_pays(rows, cols) && work_bytes >= matern_scratch_bytes(true) &&
-      entry_table_applies(o, sigma2, beta, nu))
+      entry_table_applies(o, out_t, sigma2, beta, nu))
     return d_work;
   if (o.compute == BK_F64 && o.d_cosh_table == nullptr && work_bytes >= kDecayTableBytes)
     o.d_cosh_table = (double*)d_work;
@@ -344,7 +344,7 @@ bk_status bk_matern_tile_ws(const double* locs, int64_t n, double sigma2, double
   if (n == 0) return BK_OK;
   if (locs == nullptr) return set_error(BK_ERR_INVALID_ARG, "locs is NULL");
   cudaStream_t s = (cudaStream_t)stream;
-  void* const table = matern_scratch(o, n, n, sigma2, beta, nu, d_work, work_bytes);
+  void* const table = matern_scratch(o, dtype, n, n, sigma2, beta, nu, d_work, work_bytes);
   const cudaError_t e =
       (table != nullptr)
           ? launch_matern_sym_table(locs, n, sigma2, beta, nu, out, ld, dtype, o.compute, table, s)
@@ -385,7 +385,7 @@ bk_status bk_matern_tile2_ws(const double* locs1, int64_t m, const double* locs2
   if (locs1 == nullptr || locs2 == nullptr)
     return set_error(BK_ERR_INVALID_ARG, "locs1 and locs2 must be non-NULL");
   cudaStream_t s = (cudaStream_t)stream;
-  void* const table = matern_scratch(o, m, n, sigma2, beta, nu, d_work, work_bytes);
+  void* const table = matern_scratch(o, dtype, m, n, sigma2, beta, nu, d_work, work_bytes);
   const cudaError_t e =
       (table != nullptr)
           ? launch_matern_block_table(locs1, m, locs2, n, sigma2, beta, nu, out, ld, dtype,

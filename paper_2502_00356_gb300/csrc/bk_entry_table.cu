@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
 // ---- batched: every instance's constants, tables and tiles in three launches
 __global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_desc* __restrict__ descs,
                                                              const int64_t* __restrict__ sizes,
-                                                             int count, BatchInstance* __restrict__ inst,
+                                                             int count, bool f32,
+                                                             BatchInstance* __restrict__ inst,
                                                              unsigned long long* __restrict__ next) {
   asm volatile("griddepcontrol.launch_dependents;");
   const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
@@ -72,7 +73,7 @@ __global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_des
   b.out = d.out;
   b.n = ok ? d.n : 0;
   b.ld = d.ld;
-  b.table = ok && entry_table_size(d.n, d.n) && tab_domain(d.sigma2, d.beta, d.nu);
+  b.table = ok && entry_table_size(d.n, d.n) && tab_domain(f32, d.sigma2, d.beta, d.nu);
   b.mp = matern_params(d.sigma2, d.beta, d.nu);
   inst[k] = b;
 }
@@ -147,9 +148,9 @@ size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kStride : TabLayo
 // keeps the rule, so that a matrix is the same wherever it is stored.
 bool entry_table_pays(int64_t rows, int64_t cols) { return entry_table_size(rows, cols); }
 
-bool entry_table_applies(const bk_opts& o, double sigma2, double beta, double nu) {
+bool entry_table_applies(const bk_opts& o, bk_dtype out_t, double sigma2, double beta, double nu) {
   return o.d_counters == nullptr && o.window != BK_WIN_FIXED && o.series_below == 0.0 &&
-         o.search_f64 == 0 && tab_domain(sigma2, beta, nu);
+         o.search_f64 == 0 && tab_domain(o.compute == BK_F32 && out_t == BK_F32, sigma2, beta, nu);
 }
 
 namespace {
@@ -280,7 +281,7 @@ cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* desc
                                  bk_dtype out_t, int64_t limit, int warps, int ctas_per_sm, int chunk,
                                  cudaStream_t s) {
   batched_params_kernel<<<(unsigned)((b.count + 127) / 128), 128, 0, s>>>(
-      descs, b.sizes, b.count, (BatchInstance*)b.instances, b.next);
+      descs, b.sizes, b.count, f32, (BatchInstance*)b.instances, b.next);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (f32) return launch_batched_table_t<true, float>(b, limit, warps, ctas_per_sm, chunk, s);

@@ -105,10 +105,11 @@ constexpr int kTabNodes = 485;                  // tau = -24 .. 6.25 in steps of
 
 // Whether (sigma^2, beta, nu) are inside the tables' domain: orders for which
 // the node grid holds the integral, and scales that keep every value, the FP32
-// squared distances included, a normal number.
-__host__ __device__ inline bool tab_domain(double sigma2, double beta, double nu) {
+// squared distances and coefficients included, a normal number.
+constexpr double kTabMax32 = 0x1p50;  // the largest value of an FP32 record
+__host__ __device__ inline bool tab_domain(bool f32, double sigma2, double beta, double nu) {
   return nu >= 0.02 && nu <= 10.0 && beta >= 1e-8 && beta <= 1e8 && sigma2 >= 1e-20 &&
-         sigma2 <= 1e20;
+         sigma2 <= (f32 ? kTabMax32 : 1e20);
 }
 
 // Whether a matrix of rows x cols entries is worth a table (see
@@ -336,7 +337,7 @@ __device__ __forceinline__ void tab_record(int bin, double nu, unsigned e0, doub
     // in units of the scaled square, in which the interval's width is 2^w
     const int w = o + kTabQ0 - tab_scale(ib).odd - m;
     const double iw = __hiloint2double((1023 - w) << 20, 0);
-    const bool ok = f >= 0.0f && f <= 0x1p50f;  // (subnormal values keep their absolute accuracy)
+    const bool ok = f >= 0.0f && f <= (float)kTabMax32;  // (subnormal values keep their absolute accuracy)
     reinterpret_cast<float4*>(table)[bin] = make_float4(ok ? f : __int_as_float(0x7fc00000), (float)(a1 * iw),
                                                         (float)(a2 * (iw * iw)), (float)(a3 * (iw * iw * iw)));
   } else {

@@ -152,7 +152,7 @@ bk_status bk_matern_tile_host(const double* h_locs, int64_t n, double sigma2, do
 
   char* ws = (char*)d_work;
   double* d_locs = (double*)(ws + L.locs);
-  void* const table = matern_scratch(o, n, n, sigma2, beta, nu, ws + L.scratch, L.matrix - L.scratch);
+  void* const table = matern_scratch(o, dtype, n, n, sigma2, beta, nu, ws + L.scratch, L.matrix - L.scratch);
   const size_t elem = dtype == BK_F64 ? sizeof(double) : sizeof(float);
   cudaStream_t s = (cudaStream_t)stream;
 

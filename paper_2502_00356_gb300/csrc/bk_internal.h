@@ -66,7 +66,7 @@ size_t entry_table_bytes(bool f32);
 // Whether a matrix of this size is worth a table, and whether the options and
 // parameters are inside the tables' domain.
 bool entry_table_pays(int64_t rows, int64_t cols);
-bool entry_table_applies(const bk_opts& o, double sigma2, double beta, double nu);
+bool entry_table_applies(const bk_opts& o, bk_dtype out_t, double sigma2, double beta, double nu);
 // A batch of matrices with tables (bk_batched.cu's plans): device arrays of
 // the plan, `instances` of batched_instance_bytes() and `tables` of
 // entry_table_bytes() per instance, prefix sums over tiles of 64.
@@ -90,7 +90,7 @@ int batched_table_max_ctas(bool f32, bk_dtype out_t, int warps);
 // when it fits and the caller gave none.
 constexpr size_t kDecayTableBytes = (size_t)BK_COSH_TABLE_LEN * sizeof(double);
 size_t matern_scratch_bytes(bool table);
-void* matern_scratch(bk_opts& o, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
+void* matern_scratch(bk_opts& o, bk_dtype out_t, int64_t rows, int64_t cols, double sigma2, double beta, double nu,
                      void* d_work, size_t work_bytes);
 // The writers of launch_matern_sym_* and launch_matern_block_* with a table in
 // device memory (16-byte aligned, entry_table_bytes of the records: FP32 when

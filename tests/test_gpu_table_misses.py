@@ -87,3 +87,19 @@ def test_a_matrix_is_the_same_in_host_memory(dev, n, pad, dtype):
     bk.bk_matern_tile_host(torch.as_tensor(L).pin_memory(), 0.9, 0.1, 1.3, got, work)
     torch.cuda.synchronize()
     assert torch.equal(got[:, :n], want.cpu()) and bool((got[:, n:] == -1.0).all())
+
+
+@pytest.mark.parametrize("sigma2,table", [(2.0 ** 50, True), (2.0 ** 50 * 1.001, False), (1e19, False)])
+def test_fp32_tables_hold_values_up_to_2_to_the_50(dev, sigma2, table):
+    """A larger sigma^2 takes the writer without a table, which leaves the scratch as
+    it was, instead of a table whose records near x = 0 hold nothing."""
+    n = 800
+    L = grid(n, 9, dev)
+    out = torch.empty((n, n), dtype=torch.float32, device=dev)
+    work = torch.full((bk.lib().bk_matern_workspace(n, n),), 0xA5, dtype=torch.uint8, device=dev)
+    assert bk.lib().bk_matern_tile_ws(L.data_ptr(), n, sigma2, 0.1, 1.5, out.data_ptr(), n, bk.BK_F32, None, work.data_ptr(),
+                                      work.numel(), torch.cuda.current_stream().cuda_stream or None) == bk.BK_OK
+    want = bk.bk_matern_tile(L, sigma2, 0.1, 1.5, opts=direct())
+    torch.cuda.synchronize()
+    assert bool((work != 0xA5).any()) == table
+    assert bool(((out.double() - want).abs() <= 2e-6 * want).all())
