@@ -37,11 +37,19 @@ struct BatchSmem {
 
 // Persistent kernel: each CTA repeatedly takes `chunk` consecutive tiles from
 // *next (scratch, zeroed before the launch) until `limit` tiles are taken.
-template <class Form, typename OutT, int WARPS>
+// kChosen: only the instances with direct[k] != 0 (a plan with entry tables;
+// launched while the kernels that write direct and the tables may still run).
+template <class Form, typename OutT, int WARPS, bool kChosen>
 __global__ void __launch_bounds__(WARPS * 32, Form::kMinBlocks * 8 / WARPS) matern_batched_kernel(
     const Form form, const bk_matern_desc* __restrict__ descs, int count, const int64_t* __restrict__ prefix,
     const int64_t* __restrict__ sizes, int64_t limit, unsigned long long* __restrict__ next,
-    int chunk, unsigned long long* __restrict__ ctr, const double* __restrict__ wnu_tabs) {
+    int chunk, unsigned long long* __restrict__ ctr, const double* wnu_tabs, int64_t wnu_stride, const int* direct) {
+  if constexpr (kChosen) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    int any = 0;
+    for (int k = (int)threadIdx.x; k < count; k += WARPS * 32) any |= direct[k];
+    if (!__syncthreads_or(any)) return;
+  }
   __shared__ BatchSmem<OutT> sm;
   __shared__ double s_tab[Form::kStageTable ? kExpTabSize : 1];
   const Form f = bind_table(form, s_tab);
@@ -57,6 +65,13 @@ __global__ void __launch_bounds__(WARPS * 32, Form::kMinBlocks * 8 / WARPS) mate
     const int64_t end = min(base + (int64_t)chunk, limit);
     for (int64_t w = base; w < end; ++w) {
       const int k = find_instance(prefix, count, w);
+      if constexpr (kChosen) {
+        if (!direct[k]) {  // past all of this instance's tiles
+          if (threadIdx.x == 0) atomicMax(next, (unsigned long long)__ldg(prefix + k + 1));
+          w = min(__ldg(prefix + k + 1), end) - 1;
+          continue;
+        }
+      }
       if (k != cur) {
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -73,7 +88,7 @@ __global__ void __launch_bounds__(WARPS * 32, Form::kMinBlocks * 8 / WARPS) mate
           sm.n = d.n;
           sm.ld = d.ld;
           sm.mp = matern_params(d.sigma2, d.beta, d.nu);  // a1, once per instance run
-          sm.wnu = (wnu_tabs != nullptr) ? wnu_tabs + (int64_t)k * kCoshTabSize : nullptr;
+          sm.wnu = (wnu_tabs != nullptr) ? wnu_tabs + k * wnu_stride : nullptr;
         }
         __syncthreads();
         cur = k;
@@ -120,10 +135,16 @@ struct bk_plan {
   int64_t total_tiles;
   int64_t* d_prefix;               // count + 1 tile offsets (device)
   int64_t* d_sizes;                // count instance sizes (device)
-  unsigned long long* d_next;      // tile counter (device scratch)
+  unsigned long long* d_next;      // two tile counters (device scratch)
   double* d_wnu;                   // count x kCoshTabSize: e^{-2 nu h} per instance, or null
-  void* d_inst;                    // with entry tables: the instances' constants, else null
-  void* d_tables;                  // their tables
+  // with entry tables (else null): tiles of 64 of the instances that may have one
+  // and their offsets, the instances' constants, their tables, and a flag for each
+  // instance that the per-entry kernel takes
+  int64_t table_tiles;
+  int64_t* d_table_prefix;
+  void* d_inst;
+  void* d_tables;
+  int* d_direct;
   int warps, ctas_per_sm, chunk;   // launch shape
   int tuned;                       // 1 when the shape came from the autotuner or its cache
   double tuned_ms;
@@ -156,10 +177,26 @@ template <class Form, typename OutT, int WARPS>
 cudaError_t launch_batched_t(const bk_plan* p, const bk_matern_desc* d, int64_t limit,
                              int ctas_per_sm, int chunk, cudaStream_t s) {
   const int grid = current_sm_count() * ctas_per_sm;
-  matern_batched_kernel<Form, OutT, WARPS><<<grid, WARPS * 32, 0, s>>>(
+  matern_batched_kernel<Form, OutT, WARPS, false><<<grid, WARPS * 32, 0, s>>>(
       make_form<Form>(p), d, p->count, p->d_prefix, p->d_sizes, limit, p->d_next, chunk, p->opts.d_counters,
-      Form::kDecayTable ? p->d_wnu : nullptr);
+      Form::kDecayTable ? p->d_wnu : nullptr, kCoshTabSize, nullptr);
   return cudaGetLastError();
+}
+
+// The instances of a plan with tables that have none, in the plan's form.
+template <class Form, typename OutT>
+cudaError_t launch_batched_rest(const bk_plan* p, const bk_matern_desc* d, int64_t limit, cudaStream_t s) {
+  const size_t stride = entry_table_bytes(p->opts.compute == BK_F32 && p->dtype == BK_F32);
+  return launch_next(matern_batched_kernel<Form, OutT, 8, true>, dim3((unsigned)(current_sm_count() * 2)), 256, s,
+                     make_form<Form>(p), d, p->count, (const int64_t*)p->d_prefix, (const int64_t*)p->d_sizes, limit,
+                     p->d_next + 1, 1, (unsigned long long*)nullptr,
+                     Form::kDecayTable ? (const double*)p->d_tables : nullptr, (int64_t)(stride / sizeof(double)),
+                     (const int*)p->d_direct);
+}
+template <class Form>
+cudaError_t launch_batched_rest(const bk_plan* p, const bk_matern_desc* d, int64_t limit, cudaStream_t s) {
+  return p->dtype == BK_F64 ? launch_batched_rest<Form, double>(p, d, limit, s)
+                            : launch_batched_rest<Form, float>(p, d, limit, s);
 }
 
 template <class Form, typename OutT>
@@ -175,8 +212,16 @@ bool plan_table_f32(const bk_plan* p) { return p->opts.compute == BK_F32 && p->d
 cudaError_t launch_batched(const bk_plan* p, const bk_matern_desc* d, int64_t limit, int warps,
                            int ctas_per_sm, int chunk, cudaStream_t s) {
   if (p->d_tables != nullptr) {
-    const BatchTable b{p->count, p->d_prefix, p->d_sizes, p->d_next, p->d_inst, p->d_tables};
-    return launch_batched_table(b, d, plan_table_f32(p), p->dtype, limit, warps, ctas_per_sm, chunk, s);
+    const BatchTable b{p->count, p->d_table_prefix, p->d_sizes, p->d_next, p->d_direct, p->d_inst, p->d_tables,
+                       p->opts.compute == BK_F64};
+    const int64_t tiles = limit < p->total_tiles
+                              ? std::max<int64_t>(1, (int64_t)((double)p->table_tiles * limit / p->total_tiles))
+                              : p->table_tiles;
+    const cudaError_t e = launch_batched_table(b, d, plan_table_f32(p), p->dtype, tiles, warps, ctas_per_sm, chunk, s);
+    if (e != cudaSuccess) return e;
+    return p->opts.window == BK_WIN_LEARNED ? launch_batched_rest<FormF32Learned>(p, d, limit, s)
+           : p->opts.compute == BK_F64      ? launch_batched_rest<FormF64>(p, d, limit, s)
+                                            : launch_batched_rest<FormF32>(p, d, limit, s);
   }
   cudaError_t e = cudaMemsetAsync(p->d_next, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
@@ -213,35 +258,35 @@ int max_ctas_per_sm(const bk_plan* p, int warps) {
   const bool f64 = (p->opts.compute == BK_F64);
   if (p->opts.window == BK_WIN_FIXED) {
     if (p->dtype == BK_F64)
-      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Fixed, double, 4>
-                        : (const void*)matern_batched_kernel<FormF64Fixed, double, 8>;
+      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Fixed, double, 4, false>
+                        : (const void*)matern_batched_kernel<FormF64Fixed, double, 8, false>;
     else
-      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Fixed, float, 4>
-                        : (const void*)matern_batched_kernel<FormF64Fixed, float, 8>;
+      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Fixed, float, 4, false>
+                        : (const void*)matern_batched_kernel<FormF64Fixed, float, 8, false>;
   } else if (f64 && p->opts.series_below > 0.0) {
     if (p->dtype == BK_F64)
-      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Series, double, 4>
-                        : (const void*)matern_batched_kernel<FormF64Series, double, 8>;
+      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Series, double, 4, false>
+                        : (const void*)matern_batched_kernel<FormF64Series, double, 8, false>;
     else
-      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Series, float, 4>
-                        : (const void*)matern_batched_kernel<FormF64Series, float, 8>;
+      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF64Series, float, 4, false>
+                        : (const void*)matern_batched_kernel<FormF64Series, float, 8, false>;
   } else if (p->opts.window == BK_WIN_LEARNED) {
     if (p->dtype == BK_F64)
-      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF32Learned, double, 4>
-                        : (const void*)matern_batched_kernel<FormF32Learned, double, 8>;
+      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF32Learned, double, 4, false>
+                        : (const void*)matern_batched_kernel<FormF32Learned, double, 8, false>;
     else
-      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF32Learned, float, 4>
-                        : (const void*)matern_batched_kernel<FormF32Learned, float, 8>;
+      fn = (warps == 4) ? (const void*)matern_batched_kernel<FormF32Learned, float, 4, false>
+                        : (const void*)matern_batched_kernel<FormF32Learned, float, 8, false>;
   } else if (p->dtype == BK_F64) {
-    if (warps == 4) fn = f64 ? (const void*)matern_batched_kernel<FormF64, double, 4>
-                             : (const void*)matern_batched_kernel<FormF32, double, 4>;
-    else fn = f64 ? (const void*)matern_batched_kernel<FormF64, double, 8>
-                  : (const void*)matern_batched_kernel<FormF32, double, 8>;
+    if (warps == 4) fn = f64 ? (const void*)matern_batched_kernel<FormF64, double, 4, false>
+                             : (const void*)matern_batched_kernel<FormF32, double, 4, false>;
+    else fn = f64 ? (const void*)matern_batched_kernel<FormF64, double, 8, false>
+                  : (const void*)matern_batched_kernel<FormF32, double, 8, false>;
   } else {
-    if (warps == 4) fn = f64 ? (const void*)matern_batched_kernel<FormF64, float, 4>
-                             : (const void*)matern_batched_kernel<FormF32, float, 4>;
-    else fn = f64 ? (const void*)matern_batched_kernel<FormF64, float, 8>
-                  : (const void*)matern_batched_kernel<FormF32, float, 8>;
+    if (warps == 4) fn = f64 ? (const void*)matern_batched_kernel<FormF64, float, 4, false>
+                             : (const void*)matern_batched_kernel<FormF32, float, 4, false>;
+    else fn = f64 ? (const void*)matern_batched_kernel<FormF64, float, 8, false>
+                  : (const void*)matern_batched_kernel<FormF32, float, 8, false>;
   }
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, fn, warps * 32, 0) != cudaSuccess)
     return 1;
@@ -302,6 +347,46 @@ void cache_store(const std::string& key, int warps, int cps, int chunk, double m
   std::fclose(f);
 }
 
+void free_tables(bk_plan* p) {
+  cudaFree(p->d_table_prefix);
+  cudaFree(p->d_inst);
+  cudaFree(p->d_direct);
+  cudaFree(p->d_tables);
+  p->d_table_prefix = nullptr;
+  p->d_inst = p->d_tables = nullptr;
+  p->d_direct = nullptr;
+}
+
+// Whether an instance of a plan with tables is worth one.  Many tables are built
+// side by side, in 2.4 us each (FP32 1.05): 300 instances of n = 300 took 741 us with
+// them and 2,263 without, in FP32 321 and 859, with the learned window 321 and 753;
+// 20 of them 88 and 176, 49 and 54, 49 and 62.  FP32 arithmetic into FP64 matrices
+// needs FP64 tables: 20 of n = 300 88 us with, 71 without (learned 65), 40 of n = 400
+// 200 and 219 (195), 40 of n = 500 212 and 310 (279).
+bool batch_instance_pays(int64_t n, const bk_opts& o, bk_dtype out_t) {
+  return n >= (o.compute == BK_F32 && out_t == BK_F64 ? 480 : 256);
+}
+// Whether a batch is worth tables: by the entries of the instances that are worth one,
+// as tables cost the call about 40 us (FP32 30).  Batches of such instances alone are
+// bound by one entry's latency without them, and gain early: one matrix of n = 750
+// 42 us with tables, 60 without (FP64), 31, 24 (FP32), 30, 21 (learned); of n = 1,000
+// 42, 92; 32, 33; 32, 30; FP32 arithmetic into FP64, n = 1,000 42, 34, n = 1,250 44,
+// 44.  Beside smaller instances, which keep the GPU busy and then take a launch of their
+// own, the larger ones' entries must be worth the tables by themselves (n = 900
+// beside 200 of n = 100: 390 us with tables, 342 without; FP32 164, 130).
+bool batch_pays(const int64_t* sizes, int32_t count, const bk_opts& o, bk_dtype out_t) {
+  constexpr double kUnit = 524288.0;  // 2^19 entries
+  const bool f32 = o.compute == BK_F32;
+  const double least = f32 ? (out_t == BK_F64 ? 3.0 * kUnit : 2.0 * kUnit) : kUnit;
+  double entries = 0.0;
+  bool smaller = false;
+  for (int32_t k = 0; k < count; ++k) {
+    if (batch_instance_pays(sizes[k], o, out_t)) entries += (double)sizes[k] * (double)sizes[k];
+    else smaller = smaller || sizes[k] > 0;
+  }
+  return entries >= (smaller ? (f32 ? 6.0 : 3.0) : 1.0) * least;
+}
+
 std::string make_key(const bk_plan* p) {
   cudaDeviceProp prop;
   std::string name = "gpu";
@@ -309,7 +394,7 @@ std::string make_key(const bk_plan* p) {
   for (char& c : name)
     if (c == ' ') c = '_';
   int bucket = 0;
-  while ((1LL << bucket) < p->total_tiles) ++bucket;
+  while ((1LL << bucket) < (p->d_tables != nullptr ? p->table_tiles : p->total_tiles)) ++bucket;
   char buf[256];
   std::snprintf(buf, sizeof(buf), "%s|out%d|compute%d|win%d|tiles2^%d%s", name.c_str(),
                 (int)p->dtype, (int)p->opts.compute, (int)p->opts.window, bucket,
@@ -337,31 +422,21 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   if (opts != nullptr) o = *opts; else o.compute = dtype;
   const bk_status st = check_opts(&o);
   if (st != BK_OK) return st;
-  // Entry tables (bk_entry_table.cuh) for the forms that have them, when some
-  // instance is worth one and they fit 1 GiB; the others then run in the same
-  // launch without.  The parameters are only known at each call.
-  bool pays = false;
-  for (int32_t k = 0; k < count; ++k) {
+  for (int32_t k = 0; k < count; ++k)
     if (sizes[k] < 0) return set_error(BK_ERR_INVALID_ARG, "sizes[%d] < 0", (int)k);
-    pays = pays || entry_table_pays(sizes[k], sizes[k]);
-  }
-  const size_t table_bytes =
-      (size_t)count * entry_table_bytes(o.compute == BK_F32 && dtype == BK_F32);
-  void *d_inst = nullptr, *d_tables = nullptr;
-  if (pays && count <= 65535 && table_bytes <= ((size_t)1 << 30) &&
-      entry_table_applies(o, dtype, 1.0, 1.0, 1.0)) {
-    if (cudaMalloc(&d_inst, (size_t)count * batched_instance_bytes()) != cudaSuccess ||
-        cudaMalloc(&d_tables, table_bytes) != cudaSuccess) {
-      (void)cudaGetLastError();  // without them the kernel evaluates every entry itself
-      cudaFree(d_inst);
-      d_inst = d_tables = nullptr;
-    }
-  }
-  const int64_t edge = d_tables != nullptr ? 64 : kTile;
-  std::vector<int64_t> prefix((size_t)count + 1, 0);
+  std::vector<int64_t> prefix((size_t)count + 1, 0), table_prefix((size_t)count + 1, 0);
+  // Entry tables (bk_entry_table.cuh) for the forms that have them, where the batch
+  // is worth them and they fit 1 GiB.  The parameters are only known at each call:
+  // instances outside the tables' domain, and those too small for one, are the
+  // per-entry kernel's.
+  const bool table_f32 = o.compute == BK_F32 && dtype == BK_F32;
+  const size_t table_bytes = (size_t)count * entry_table_bytes(table_f32);
+  const bool tables = count <= 65535 && table_bytes <= ((size_t)1 << 30) &&
+                      entry_table_applies(o, dtype, 1.0, 1.0, 1.0) && batch_pays(sizes, count, o, dtype);
   for (int32_t k = 0; k < count; ++k) {
-    const int64_t nb = (sizes[k] + edge - 1) / edge;
+    const int64_t nb = (sizes[k] + kTile - 1) / kTile, nt = batch_instance_pays(sizes[k], o, dtype) ? (sizes[k] + 63) / 64 : 0;
     prefix[(size_t)k + 1] = prefix[(size_t)k] + nb * (nb + 1) / 2;
+    table_prefix[(size_t)k + 1] = table_prefix[(size_t)k] + nt * (nt + 1) / 2;
   }
   bk_plan* p = new bk_plan();
   p->count = count;
@@ -372,8 +447,11 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   p->d_sizes = nullptr;
   p->d_next = nullptr;
   p->d_wnu = nullptr;
-  p->d_inst = d_inst;
-  p->d_tables = d_tables;
+  p->table_tiles = table_prefix.back();
+  p->d_table_prefix = nullptr;
+  p->d_inst = nullptr;
+  p->d_tables = nullptr;
+  p->d_direct = nullptr;
   p->warps = 8;
   p->chunk = 1;
   p->tuned = 0;
@@ -381,16 +459,28 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   cudaError_t e = cudaGetDevice(&p->device);
   if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_prefix, prefix.size() * sizeof(int64_t));
   if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_sizes, (size_t)count * sizeof(int64_t));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_next, sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_next, 2 * sizeof(unsigned long long));
   if (e == cudaSuccess)
     e = cudaMemcpy(p->d_prefix, prefix.data(), prefix.size() * sizeof(int64_t),
                    cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(p->d_sizes, sizes, (size_t)count * sizeof(int64_t), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && tables) {
+    const size_t offsets = table_prefix.size() * sizeof(int64_t);
+    if (cudaMalloc((void**)&p->d_table_prefix, offsets) != cudaSuccess ||
+        cudaMalloc(&p->d_inst, (size_t)count * batched_instance_bytes()) != cudaSuccess ||
+        cudaMalloc((void**)&p->d_direct, (size_t)count * sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&p->d_tables, table_bytes) != cudaSuccess) {
+      (void)cudaGetLastError();  // without them the per-entry kernel takes every instance
+      free_tables(p);
+    } else {
+      e = cudaMemcpy(p->d_table_prefix, table_prefix.data(), offsets, cudaMemcpyHostToDevice);
+    }
+  }
   // per-instance tables of e^{-2 nu h} for the searched-window FP64 forms
   // (without them, or for more than 4,096 instances, the kernel computes the
   // values itself)
-  if (e == cudaSuccess && d_tables == nullptr && o.compute == BK_F64 && o.window != BK_WIN_FIXED &&
+  if (e == cudaSuccess && p->d_tables == nullptr && o.compute == BK_F64 && o.window != BK_WIN_FIXED &&
       o.window != BK_WIN_LEARNED && count <= 4096) {
     if (cudaMalloc((void**)&p->d_wnu, (size_t)count * kCoshTabSize * sizeof(double)) != cudaSuccess) {
       (void)cudaGetLastError();
@@ -401,8 +491,7 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
     cudaFree(p->d_prefix);
     cudaFree(p->d_sizes);
     cudaFree(p->d_next);
-    cudaFree(p->d_inst);
-    cudaFree(p->d_tables);
+    free_tables(p);
     delete p;
     return (e == cudaErrorMemoryAllocation) ? set_error(BK_ERR_NOMEM, "plan: out of device memory")
                                             : check_cuda(e, "bk_batched_plan_create");
@@ -429,8 +518,7 @@ bk_status bk_batched_plan_destroy(bk_plan* plan) {
   cudaFree(plan->d_sizes);
   cudaFree(plan->d_next);
   cudaFree(plan->d_wnu);
-  cudaFree(plan->d_inst);
-  cudaFree(plan->d_tables);
+  free_tables(plan);
   delete plan;
   return BK_OK;
 }

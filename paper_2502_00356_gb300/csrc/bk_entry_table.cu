@@ -56,45 +56,48 @@ __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
 
 // ---- batched: every instance's constants, tables and tiles in three launches
 __global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_desc* __restrict__ descs,
-                                                             const int64_t* __restrict__ sizes,
-                                                             int count, bool f32,
-                                                             BatchInstance* __restrict__ inst,
-                                                             unsigned long long* __restrict__ next) {
+                                                             const __grid_constant__ BatchTable t, bool f32,
+                                                             BatchInstance* __restrict__ inst) {
   asm volatile("griddepcontrol.launch_dependents;");
   const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (k == 0) *next = 0ull;
-  if (k >= count) return;
+  if (k == 0) t.next[0] = t.next[1] = 0ull;
+  if (k >= t.count) return;
   const bk_matern_desc d = descs[k];
   // a descriptor that does not match the plan is skipped (n = 0)
-  const bool ok = d.n == sizes[k] && d.ld >= d.n && d.locs != nullptr && d.out != nullptr &&
+  const bool ok = d.n == t.sizes[k] && d.ld >= d.n && d.locs != nullptr && d.out != nullptr &&
                   d.beta > 0.0 && d.nu > 0.0 && d.sigma2 >= 0.0;
   BatchInstance b;
   b.locs = d.locs;
   b.out = d.out;
   b.n = ok ? d.n : 0;
   b.ld = d.ld;
-  b.table = ok && entry_table_size(d.n, d.n) && tab_domain(f32, d.sigma2, d.beta, d.nu);
+  b.table = ok && t.prefix[k + 1] > t.prefix[k] && tab_domain(f32, d.sigma2, d.beta, d.nu);
+  t.direct[k] = ok && !b.table;
   b.mp = matern_params(d.sigma2, d.beta, d.nu);
   inst[k] = b;
 }
 
 template <bool F32>
 __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
-    const BatchInstance* inst, unsigned char* __restrict__ tables) {  // (inst: not read-only, load_record)
+    const BatchInstance* inst, unsigned char* __restrict__ tables, bool decays) {  // (inst: not read-only, load_record)
   __shared__ TabBuildSmem sm;
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
   const BatchInstance& b = inst[blockIdx.y];
-  if (!b.table) {
-    if (!F32 && blockIdx.x == 0 && threadIdx.x == 0)
-      *reinterpret_cast<double*>(tables + (size_t)blockIdx.y * TabLayout<F32>::kStride) = -1.0;
+  const MaternParams mp = b.mp;
+  if (!b.table) {  // for the per-entry kernel: the plain form's e^{-2 nu h}
+    if constexpr (!F32) {
+      double* const decay = reinterpret_cast<double*>(tables + (size_t)blockIdx.y * TabLayout<F32>::kStride);
+      for (int i = (int)(blockIdx.x * kTabThreads + threadIdx.x); decays && b.n > 0 && i < kCoshTabSize; i += (int)gridDim.x * kTabThreads)
+        decay[i] = decay_entry(mp.nu, i, kExp2Tab);
+    }
     return;
   }
-  const MaternParams mp = b.mp;
   tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, b.n <= kTabScan, b.locs, b.n, b.locs, b.n,
                        tables + (size_t)blockIdx.y * TabLayout<F32>::kStride + TabLayout<F32>::kFront);
 }
 
-// Persistent kernel as matern_batched_kernel, in tiles of 64.
+// Persistent kernel as matern_batched_kernel, in tiles of 64 of the instances that
+// may have a table; one that has none (parameters outside the domain) is passed over.
 template <bool F32, typename OutT, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_kernel(
     const BatchInstance* inst, int count, const int64_t* __restrict__ prefix,
@@ -124,11 +127,15 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
               reinterpret_cast<const long long*>(inst + k)[threadIdx.x];
         __syncthreads();
       }
+      if (!cur.table) {
+        if (threadIdx.x == 0) atomicMax(next, (unsigned long long)__ldg(prefix + k + 1));
+        w = min(__ldg(prefix + k + 1), end) - 1;
+        continue;
+      }
       int64_t I, J;
       tri_tile(w - __ldg(prefix + k), I, J);
       tab_tile<F32, OutT, true, WARPS>(sm, tables + (size_t)k * TabLayout<F32>::kStride + TabLayout<F32>::kFront,
-                                       cur.locs, cur.n, cur.locs, cur.n, I, J, cur.mp, (OutT*)cur.out, cur.ld, 0, kTabTile,
-                                       cur.table != 0);
+                                       cur.locs, cur.n, cur.locs, cur.n, I, J, cur.mp, (OutT*)cur.out, cur.ld);
     }
   }
 }
@@ -167,23 +174,6 @@ int tile_width(int64_t ntiles, bool host, int64_t column_bytes) {
   if (ntiles >= 4 * sms) return kTabTile;
   if (!host) return kTabTile / 4;
   return column_bytes % 32 != 0 && 2 * ntiles >= 3 * sms ? kTabTile : kTabTile / 2;
-}
-
-// Launches a kernel so that it may be scheduled while the one before it still
-// runs (it waits for that kernel's end itself): the launch's latency, about 3 us,
-// is hidden (batches of 3: 77.5 -> 70.9 us in FP32, 90.9 -> 86.7 in FP64).
-template <typename... P, typename... A>
-cudaError_t launch_next(void (*kernel)(P...), dim3 grid, int block, cudaStream_t s, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
 }
 
 template <typename... P, typename... A>
@@ -268,7 +258,7 @@ cudaError_t launch_batched_table_t(const BatchTable& b, int64_t limit, int warps
   // node weights, once per block, stay a small part of it.
   const int sms = current_sm_count(), share = b.count < sms / 4 ? sms / b.count : 4;
   const cudaError_t e = launch_next(batched_table_kernel<F32>, dim3((unsigned)share, (unsigned)b.count),
-                                    kTabThreads, s, (const BatchInstance*)b.instances, (unsigned char*)b.tables);
+                                    kTabThreads, s, (const BatchInstance*)b.instances, (unsigned char*)b.tables, b.decay);
   if (e != cudaSuccess) return e;
   return launch_next(warps == 4 ? matern_batched_table_kernel<F32, OutT, 4> : matern_batched_table_kernel<F32, OutT, 8>,
                      dim3((unsigned)(sms * ctas_per_sm)), warps * 32, s, (const BatchInstance*)b.instances, b.count,
@@ -281,7 +271,7 @@ cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* desc
                                  bk_dtype out_t, int64_t limit, int warps, int ctas_per_sm, int chunk,
                                  cudaStream_t s) {
   batched_params_kernel<<<(unsigned)((b.count + 127) / 128), 128, 0, s>>>(
-      descs, b.sizes, b.count, f32, (BatchInstance*)b.instances, b.next);
+      descs, b, f32, (BatchInstance*)b.instances);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (f32) return launch_batched_table_t<true, float>(b, limit, warps, ctas_per_sm, chunk, s);

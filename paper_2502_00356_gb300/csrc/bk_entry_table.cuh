@@ -792,23 +792,21 @@ __device__ __forceinline__ OutT tab_direct(const double* __restrict__ locs1, int
 // block of WARPS warps: lane i of warp w takes rows i and i + 32 of columns w,
 // w + WARPS, ..., two rows at a time so that the loads of one entry overlap the
 // arithmetic of the other.  kSym: the transposed block (J, I) is written too.
-// use_table false: every entry by the direct evaluation.  part, width: the block
-// takes columns part * width .. + width - 1 only (width 16, 32 or 64: tile_width),
+// part, width: the block takes columns part * width .. + width - 1 only (width 16, 32 or 64: tile_width),
 // where whole tiles would leave SMs without a block.
 template <bool F32, typename OutT, bool kSym, int WARPS>
 __device__ __forceinline__ void tab_tile(TabTileSmem<F32, OutT>& sm, const unsigned char* table,
                                          const double* __restrict__ locs1, int64_t m,
                                          const double* __restrict__ locs2, int64_t n, int64_t I,
                                          int64_t J, const MaternParams& mp, OutT* __restrict__ out,
-                                         int64_t ld, int part = 0, int width = kTabTile,
-                                         bool use_table = true) {
+                                         int64_t ld, int part = 0, int width = kTabTile) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t r0 = I * kTabTile, c0 = J * kTabTile;
   const bool in0 = r0 + lane < m, in1 = r0 + lane + 32 < m;
   const int cb = part * width, cw = cb + warp;  // the part's first column, the warp's
   const int cols = (int)(n - c0 < cb + width ? n - c0 : cb + width);
   OutT* const p0 = out + (r0 + lane) + (c0 + cw) * ld;
-  use_table = use_table && tab_stage<F32, WARPS * 32>(sm.pts, locs1, m, locs2, n, r0, c0, mp, table);
+  const bool use_table = tab_stage<F32, WARPS * 32>(sm.pts, locs1, m, locs2, n, r0, c0, mp, table);
   __syncthreads();
   const auto a0 = sm.pts.p[lane], a1 = sm.pts.p[lane + 32];
   NanSeen nan;

@@ -69,14 +69,19 @@ bool entry_table_pays(int64_t rows, int64_t cols);
 bool entry_table_applies(const bk_opts& o, bk_dtype out_t, double sigma2, double beta, double nu);
 // A batch of matrices with tables (bk_batched.cu's plans): device arrays of
 // the plan, `instances` of batched_instance_bytes() and `tables` of
-// entry_table_bytes() per instance, prefix sums over tiles of 64.
+// entry_table_bytes() per instance, prefix sums over the tiles of 64 of the
+// instances that may have a table, two tile counters (the second of the per-entry
+// kernel), and what that kernel is to take: direct[k] != 0 for valid instances
+// without a table, whose e^{-2 nu h} then stand in place of the table (decay).
 struct BatchTable {
   int count;
   const int64_t* prefix;
   const int64_t* sizes;
   unsigned long long* next;
+  int* direct;
   void* instances;
   void* tables;
+  bool decay;
 };
 size_t batched_instance_bytes();
 cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* descs, bool f32,
