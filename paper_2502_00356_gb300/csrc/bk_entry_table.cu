@@ -54,46 +54,49 @@ __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
   tab_tile<F32, OutT, kSym, 8>(sm, table, locs1, m, locs2, n, I, J, mp, out, ld, (int)part, width);
 }
 
-// ---- batched: every instance's constants, tables and tiles in three launches
-__global__ void __launch_bounds__(128) batched_params_kernel(const bk_matern_desc* __restrict__ descs,
-                                                             const __grid_constant__ BatchTable t, bool f32,
-                                                             BatchInstance* __restrict__ inst) {
-  asm volatile("griddepcontrol.launch_dependents;");
-  const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  if (k == 0) t.next[0] = t.next[1] = 0ull;
-  if (k >= t.count) return;
-  const bk_matern_desc d = descs[k];
-  // a descriptor that does not match the plan is skipped (n = 0)
-  const bool ok = d.n == t.sizes[k] && d.ld >= d.n && d.locs != nullptr && d.out != nullptr &&
-                  d.beta > 0.0 && d.nu > 0.0 && d.sigma2 >= 0.0;
-  BatchInstance b;
-  b.locs = d.locs;
-  b.out = d.out;
-  b.n = ok ? d.n : 0;
-  b.ld = d.ld;
-  b.table = ok && t.prefix[k + 1] > t.prefix[k] && tab_domain(f32, d.sigma2, d.beta, d.nu);
-  t.direct[k] = ok && !b.table;
-  b.mp = matern_params(d.sigma2, d.beta, d.nu);
-  inst[k] = b;
-}
-
+// ---- batched: every instance's constants and table in one launch, all tiles in
+// the next, instances without a table in a third (bk_batched.cu) ----
+// Block (b, k): instance k's constants, which its first block also stores, and its
+// share of the instance's table.  (A kernel of their own for the constants cost 2 us.)
 template <bool F32>
 __global__ void __launch_bounds__(kTabThreads) batched_table_kernel(
-    const BatchInstance* inst, unsigned char* __restrict__ tables, bool decays) {  // (inst: not read-only, load_record)
+    const bk_matern_desc* __restrict__ descs, const __grid_constant__ BatchTable t) {
   __shared__ TabBuildSmem sm;
-  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
-  const BatchInstance& b = inst[blockIdx.y];
-  const MaternParams mp = b.mp;
+  __shared__ BatchInstance b;
+  asm volatile("griddepcontrol.launch_dependents;");
+  const int k = (int)blockIdx.y;
+  if (threadIdx.x == 0) {
+    const bk_matern_desc d = descs[k];
+    // a descriptor that does not match the plan is skipped (n = 0)
+    const bool ok = d.n == t.sizes[k] && d.ld >= d.n && d.locs != nullptr && d.out != nullptr &&
+                    d.beta > 0.0 && d.nu > 0.0 && d.sigma2 >= 0.0;
+    b.locs = d.locs;
+    b.out = d.out;
+    b.n = ok ? d.n : 0;
+    b.ld = d.ld;
+    b.table = ok && t.prefix[k + 1] > t.prefix[k] && tab_domain(F32, d.sigma2, d.beta, d.nu);
+    b.mp = matern_params(d.sigma2, d.beta, d.nu);
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    constexpr int kWords = (int)(sizeof(BatchInstance) / 8);
+    if (threadIdx.x < kWords)
+      reinterpret_cast<long long*>((BatchInstance*)t.instances + k)[threadIdx.x] =
+          reinterpret_cast<const long long*>(&b)[threadIdx.x];
+    if (threadIdx.x == 0) t.direct[k] = b.n > 0 && !b.table;
+    if (k == 0 && threadIdx.x < 2) t.next[threadIdx.x] = 0ull;
+  }
+  unsigned char* const table = (unsigned char*)t.tables + (size_t)k * TabLayout<F32>::kStride;
   if (!b.table) {  // for the per-entry kernel: the plain form's e^{-2 nu h}
     if constexpr (!F32) {
-      double* const decay = reinterpret_cast<double*>(tables + (size_t)blockIdx.y * TabLayout<F32>::kStride);
-      for (int i = (int)(blockIdx.x * kTabThreads + threadIdx.x); decays && b.n > 0 && i < kCoshTabSize; i += (int)gridDim.x * kTabThreads)
-        decay[i] = decay_entry(mp.nu, i, kExp2Tab);
+      for (int i = (int)(blockIdx.x * kTabThreads + threadIdx.x); t.decay && b.n > 0 && i < kCoshTabSize;
+           i += (int)gridDim.x * kTabThreads)
+        reinterpret_cast<double*>(table)[i] = decay_entry(b.mp.nu, i, kExp2Tab);
     }
     return;
   }
-  tab_build_block<F32>(sm, mp, (int)blockIdx.x, (int)gridDim.x, b.n <= kTabScan, b.locs, b.n, b.locs, b.n,
-                       tables + (size_t)blockIdx.y * TabLayout<F32>::kStride + TabLayout<F32>::kFront);
+  tab_build_block<F32>(sm, b.mp, (int)blockIdx.x, (int)gridDim.x, b.n <= kTabScan, b.locs, b.n, b.locs, b.n,
+                       table + TabLayout<F32>::kFront);
 }
 
 // Persistent kernel as matern_batched_kernel, in tiles of 64 of the instances that
@@ -252,13 +255,13 @@ size_t batched_instance_bytes() { return sizeof(BatchInstance); }
 namespace {
 
 template <bool F32, typename OutT>
-cudaError_t launch_batched_table_t(const BatchTable& b, int64_t limit, int warps, int ctas_per_sm,
-                                   int chunk, cudaStream_t s) {
+cudaError_t launch_batched_table_t(const BatchTable& b, const bk_matern_desc* descs, int64_t limit, int warps,
+                                   int ctas_per_sm, int chunk, cudaStream_t s) {
   // The instances' tables in one wave of blocks; at least four each, so that the
   // node weights, once per block, stay a small part of it.
   const int sms = current_sm_count(), share = b.count < sms / 4 ? sms / b.count : 4;
-  const cudaError_t e = launch_next(batched_table_kernel<F32>, dim3((unsigned)share, (unsigned)b.count),
-                                    kTabThreads, s, (const BatchInstance*)b.instances, (unsigned char*)b.tables, b.decay);
+  batched_table_kernel<F32><<<dim3((unsigned)share, (unsigned)b.count), kTabThreads, 0, s>>>(descs, b);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return launch_next(warps == 4 ? matern_batched_table_kernel<F32, OutT, 4> : matern_batched_table_kernel<F32, OutT, 8>,
                      dim3((unsigned)(sms * ctas_per_sm)), warps * 32, s, (const BatchInstance*)b.instances, b.count,
@@ -270,13 +273,9 @@ cudaError_t launch_batched_table_t(const BatchTable& b, int64_t limit, int warps
 cudaError_t launch_batched_table(const BatchTable& b, const bk_matern_desc* descs, bool f32,
                                  bk_dtype out_t, int64_t limit, int warps, int ctas_per_sm, int chunk,
                                  cudaStream_t s) {
-  batched_params_kernel<<<(unsigned)((b.count + 127) / 128), 128, 0, s>>>(
-      descs, b, f32, (BatchInstance*)b.instances);
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  if (f32) return launch_batched_table_t<true, float>(b, limit, warps, ctas_per_sm, chunk, s);
-  if (out_t == BK_F32) return launch_batched_table_t<false, float>(b, limit, warps, ctas_per_sm, chunk, s);
-  return launch_batched_table_t<false, double>(b, limit, warps, ctas_per_sm, chunk, s);
+  if (f32) return launch_batched_table_t<true, float>(b, descs, limit, warps, ctas_per_sm, chunk, s);
+  if (out_t == BK_F32) return launch_batched_table_t<false, float>(b, descs, limit, warps, ctas_per_sm, chunk, s);
+  return launch_batched_table_t<false, double>(b, descs, limit, warps, ctas_per_sm, chunk, s);
 }
 
 int batched_table_max_ctas(bool f32, bk_dtype out_t, int warps) {
