@@ -459,7 +459,9 @@ bk_status bk_gaussian_loglik(double* a, int64_t n, int64_t ld, const double* z, 
  * finite, or that reaches 2^{s_i + s_j} (2^{2 s_i} the power of four above a_ii,
  * so between 1 and 4 times sqrt(a_ii a_jj)), counts as not positive definite, as
  * does one with a pivot <= 0 or with a row of L longer than its diagonal entry
- * allows.  Two launches per 64 rows.  d_work == NULL or too small: bk_gaussian_loglik. */
+ * allows.  The kernels' waits for their own copies and products are bounded; one
+ * that gave up (about a second; never seen) gives NaN too, and adds 2^32 instead of 1
+ * to BK_CTR_FAIL.  Two launches per 64 rows.  d_work == NULL or too small: bk_gaussian_loglik. */
 size_t bk_gaussian_loglik_workspace(int64_t n);
 bk_status bk_gaussian_loglik_ws(double* a, int64_t n, int64_t ld, const double* z, double* y,
                                 double* out, const bk_opts* opts, void* d_work, size_t work_bytes,

@@ -67,9 +67,11 @@ constexpr int kEpiCols = kNB / (kEpiWarps / 4);            // columns of an epil
 constexpr int kUpdThreads = (kEpiWarps + 2) * 32;          // epilogue, MMA, copies
 constexpr long long kWaitCycles = 2000000000LL;            // bound of every barrier wait, about 1 s
 
+constexpr int kNotPd = 1, kGaveUp = 2;   // not positive definite; a wait that gave up
+
 // The workspace.
 struct CholWork {
-  int* flag;       // not positive definite (1), or a wait that gave up (2)
+  int* flag;       // kNotPd, kGaveUp
   int* scale;      // s_i
   double* diag;    // two 64 x 64 factors, column-major: panel k's at k mod 2
   double* part;    // per panel: sum log L_ii, sum y_i^2
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(256) chol_prep_kernel(const double* __restrict
   const long long bits = __double_as_longlong(d);
   const int e = bits >> 52 ? (int)(bits >> 52) - 1023 : -1011 - __clzll(bits);  // (subnormal)
   if (bits <= 0 || e == 1024) {
-    *w.flag = 1;
+    atomicOr(w.flag, kNotPd);
     w.scale[i] = 0;
   } else {
     w.scale[i] = (e >> 1) + 1;
@@ -319,7 +321,7 @@ __device__ __forceinline__ void finish_panel(double* __restrict__ a, int64_t ld,
       const unsigned quad = 15u << (tid & 28);
       sum += __shfl_xor_sync(quad, sum, 1);
       sum += __shfl_xor_sync(quad, sum, 2);
-      if (sum > kMaxSquares) *w.flag = 1;
+      if (sum > kMaxSquares) atomicOr(w.flag, kNotPd);
     }
   }
 }
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
     }
     if (kFirst && !ok) {
       sm.bad = 1;
-      *w.flag = 1;
+      atomicOr(w.flag, kNotPd);
     }
   }
   __syncthreads();
@@ -537,7 +539,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) chol_panel_kernel(
   }
   const bool bad = sm.bad != 0;
   if ((int)blockIdx.x == row_blocks - 1) {
-    if (bad && tid == 0) *w.flag = 1;
+    if (bad && tid == 0) atomicOr(w.flag, kNotPd);
     for (int e = tid; e < kNB * kNB; e += kPanelThreads) {
       const int r = e & 63, c = e >> 6;
       double v = r == c ? 1.0 : 0.0;
@@ -762,7 +764,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
         }
         next_tile();
       }
-      if (!ok) *w.flag = 2;
+      if (!ok) atomicOr(w.flag, kGaveUp);
       // copies in flight land before the block ends
       for (int s = 0; s < kSlices && loads > 0; ++s) wait_phase(&bar.full_a[s], (uint32_t)(loads - 1) & 1u);
       for (int b = 0; b < 2; ++b)
@@ -824,7 +826,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
     }
     // products in flight end before the accumulators are given back
     if (elect_one()) {
-      if (!ok) *w.flag = 2;
+      if (!ok) atomicOr(w.flag, kGaveUp);
       tc::commit(&bar.last);
     }
     __syncwarp();
@@ -856,7 +858,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
 #pragma unroll
         for (int c = 0; c < kEpiCols; ++c) {
           long long f = 0;
-          if (c < cols && !to_fixed(__longlong_as_double(acc[c]), sr + w.scale[cb + c], f)) *w.flag = 1;
+          if (c < cols && !to_fixed(__longlong_as_double(acc[c]), sr + w.scale[cb + c], f)) atomicOr(w.flag, kNotPd);
           acc[c] = f;
         }
       }
@@ -892,7 +894,7 @@ __global__ void __launch_bounds__(kUpdThreads, 1) chol_update_kernel(
       }
       next_tile();
     }
-    if (!ok && lane == 0) *w.flag = 2;
+    if (!ok && lane == 0) atomicOr(w.flag, kGaveUp);
   }
   tc::fence_before();
   __syncthreads();
@@ -920,9 +922,9 @@ __global__ void __launch_bounds__(kPanelThreads) chol_finish_kernel(
     q += __shfl_xor_sync(0xffffffffu, q, s);
   }
   if (lane != 0) return;
-  if (*w.flag != 0) {
+  if (const int flag = *w.flag; flag != 0) {
     ld_ = q = qnan();
-    if (ctr != nullptr) atomicAdd(ctr + BK_CTR_FAIL, 1ull);
+    if (ctr != nullptr) atomicAdd(ctr + BK_CTR_FAIL, (flag & kGaveUp) != 0 ? 1ull << 32 : 1ull);
   }
   out[1] = 2.0 * ld_;
   out[2] = q;
