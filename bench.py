@@ -313,6 +313,9 @@ def _counters(bk, dev):
 
 
 def _ctr_summary(bk, c):
+    """Per-evaluation counts.  A matrix with counters is evaluated entry by entry;
+    the timed matrices come from entry tables, which count nothing, so there the
+    counts stand under "direct_evaluation"."""
     evals = max(1, int(c[bk.BK_CTR_EVALS]))
     return {"evals": int(c[bk.BK_CTR_EVALS]), "nodes_per_eval": float(c[bk.BK_CTR_NODES]) / evals,
             "fallback_rate": float(c[bk.BK_CTR_FALLBACK]) / evals,
@@ -384,8 +387,8 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
     res["fp32_matern"] = {
         "workload": f"C3: n={n3} jittered grid, beta={beta3}, nu={nu3:.4f} (U(0.3,3.5), seed 5), "
                     "FP32 out", "value": n3 * n3 / t, "unit": "entries/s", "ms": 1e3 * t,
-        "counters": cs, "roofline": write_roofline("matern_table_kernel<true, float, true>", t,
-                                                   4 * n3 * n3)}
+        "direct_evaluation": cs, "roofline": write_roofline("matern_table_kernel<true, float, true>", t,
+                                                            4 * n3 * n3)}
     sample_matrix("fp32_matern", o32, L3h, 1.0, beta3, nu3, 1_000_000, 6, 0.01)
 
     # -- C5 matrix: learned window vs searched window vs plain FP64, n = 40,000, beta = 0.1,
@@ -399,6 +402,13 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
     t_l = _time(lambda: bk.bk_matern_tile(L3, 1.0, beta5, nu5, out=o_l, opts=lo), stream, 3)
     sample_matrix("learned_matern", o_l, L3h, 1.0, beta5, nu5, 100_000, 7, 0.01)
     t_s = _time(lambda: bk.bk_matern_tile(L3, 1.0, beta5, nu5, out=o_l), stream, 3)
+    # the same two entry by entry (both searched and learned windows come from one table above)
+    od_l = bk.make_opts(learned=net, counters=c_l)
+    od_s = bk.make_opts(compute=bk.BK_F32, counters=c_l)
+    t_ld = _time(lambda: bk.bk_matern_tile(L3, 1.0, beta5, nu5, out=o_l, opts=od_l), stream, 3)
+    t_sd = _time(lambda: bk.bk_matern_tile(L3, 1.0, beta5, nu5, out=o_l, opts=od_s), stream, 3)
+    cl.update({"value": n5 * n5 / t_ld, "fp32_search_value": n5 * n5 / t_sd,
+               "learned_over_fp32_search": t_sd / t_ld})
     del o32, o_l
     torch.cuda.empty_cache()
     o64 = torch.empty((n5, n5), dtype=torch.float64, device=dev)
@@ -409,8 +419,7 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
         "workload": f"C5: n={n5} jittered grid, beta={beta5}, nu={nu5}, FP32 out",
         "value": n5 * n5 / t_l, "fp32_search_value": n5 * n5 / t_s,
         "plain_fp64_value": n5 * n5 / t_p, "unit": "entries/s",
-        "learned_over_plain": t_p / t_l, "learned_over_fp32_search": t_s / t_l,
-        "counters": cl, "fallback_rate": cl["fallback_rate"],
+        "learned_over_plain": t_p / t_l, "direct_evaluation": cl,
         "roofline": write_roofline("matern_table_kernel<true, float, true>", t_l, 4 * n5 * n5)}
     del L3
     torch.cuda.empty_cache()
@@ -465,7 +474,8 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
     locs_h = [i.locations() for i in insts]
     locs = [torch.as_tensor(h, device=dev) for h in locs_h]
     bres = {"workload": "C4: 256 instances, n log-uniform [500, 8000], sigma2 U[0.5,2], "
-                        "beta U[0.02,0.3], nu U[0.3,3], one launch replayed from a CUDA graph",
+                        "beta U[0.02,0.3], nu U[0.3,3], one call replayed from a CUDA graph; every "
+                        "instance from its entry table, in which no window is searched or predicted",
             "entries": entries}
     for name, dtype, form_opts in (("fp64", torch.float64, {}),
                                    ("fp32", torch.float32, {}),
@@ -489,7 +499,7 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
             bk.bk_matern_batched(d, plan)
         tb = _time(g.replay, stream, 2 if name == "fp64" else 5)
         bres[name] = {"value": entries / tb, "unit": "entries/s", "ms": 1e3 * tb,
-                      "plan": plan.info(), "counters": cbs}
+                      "plan": plan.info(), "direct_evaluation": cbs}
         if not form_opts:  # the allocation-free entry point on the same sweep (no plan)
             bk.bk_matern_batched_static(d, len(insts), dtype=dtype)
             ts = _time(lambda: bk.bk_matern_batched_static(d, len(insts), dtype=dtype), stream,
@@ -499,7 +509,6 @@ def measure_forms(bk, inputs, dev, stream, args, plain_rate):
             bres[name]["roofline"] = write_roofline("matern_batched_table_kernel<true, float>", tb,
                                                     4 * entries)
         if name == "learned_fp32":
-            bres[name]["fallback_rate"] = cbs["fallback_rate"]
             for k, (inst, o) in enumerate(zip(insts, outs)):
                 I, J = inputs.entry_sample(inst.n, 400, seed=1000 + k, near_fraction=0.01)
                 got = o[torch.as_tensor(J, device=dev), torch.as_tensor(I, device=dev)]
@@ -995,9 +1004,9 @@ def main():
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
             "clocks": clk.summary(), "gpu_launches": args.steps * len(NUS) * LAUNCHES_PER_MATRIX,
             "launch_ms": {str(nu): statistics.mean(v) for nu, v in zip(NUS, launch_ms)},
-            "failed_points": fails,
             "error_vs_oracle": (checks or {}).get("plain_fp64"),
-            "plain_window_fallback_rate": fallbacks / max(evals_counted, 1),
+            "direct_evaluation": {"failed_points": fails,
+                                  "window_fallback_rate": fallbacks / max(evals_counted, 1)},
             "eval_fp64": {"value": eval_rate, "unit": "K_nu evals/s",
                           "workload": "100,000 pairs, x log-uniform [1e-3,140], nu U[0.05,10]",
                           "with_grad_value": grad_rate,
