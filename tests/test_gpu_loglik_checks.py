@@ -123,3 +123,17 @@ def test_rows_at_the_end_of_their_scale_pass(dev):
     (fixed, count), (plain, _) = both(A, dev)
     # condition about 2^40: the two log determinants agree to n 2^-53 of that per pivot
     assert count == 0 and abs(fixed[1] - plain[1]) <= 1e-2 * n
+
+
+def test_small_entries_of_the_factor_by_the_fp64_factorisation(dev):
+    """A = L L^T with entries of 2^-70 below a unit diagonal: in fixed point (60
+    fraction bits) they are lost, with fp64=True the factor has them exactly."""
+    n = 130
+    A = torch.eye(n, dtype=torch.float64, device=dev)
+    for i, j in ((5, 1), (70, 3), (129, 64), (128, 127)):
+        A[i, j] = A[j, i] = 2.0 ** -70
+    z = torch.ones(n, dtype=torch.float64, device=dev)
+    a, b = A.clone(), A.clone()
+    out, plain = bk.bk_gaussian_loglik(a, z), bk.bk_gaussian_loglik(b, z, fp64=True)
+    torch.cuda.synchronize()
+    assert torch.equal(out, plain) and torch.equal(b, A) and float((a - A).abs().max()) <= 2.0 ** -59
