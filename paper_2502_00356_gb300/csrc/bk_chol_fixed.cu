@@ -144,11 +144,6 @@ __device__ __forceinline__ Limbs limbs(long long x) {
   return Limbs{l, (int)(x >> 32) + (l < 0 ? 1 : 0)};
 }
 __device__ __forceinline__ long long value(Limbs a) { return ((long long)a.h << 32) + a.l; }
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
-  long long r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
-}
 // Accumulates x y / 2^60 in two parts (high products, crossed products), rounded
 // to nearest at the end.  The products of the low words (below 4 units, of
 // either sign) are left out, except where x and y may be the same number

@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(WARPS * 32, 32 / WARPS) matern_batched_table_k
 
 size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kStride : TabLayout64::kStride; }
 
-// entry_table_size (the header): a matrix is worth a table, which costs about 13 us,
+// A matrix is worth a table, which costs about 13 us,
 // from 2^19 entries on (n = 725) in every form, as the writers without one are bound
 // by one entry's latency there.  n = 800, beta = 0.1, nu = 0.8: 27 us with it, without
 // 66 (FP64), 44 (FP32), 34 (learned); blocks of 520,000 entries 24 with it, without
@@ -156,7 +156,10 @@ size_t entry_table_bytes(bool f32) { return f32 ? TabLayout32::kStride : TabLayo
 // (n = 800: 53 and 36 us, without 75 and 49 to 61); the learned form takes 36 (38) at
 // n = 800, 47 (42) at 900, 44 (41) at 1,024, 57 (58) at 1,280, 85 (88) at 1,450, and
 // keeps the rule, so that a matrix is the same wherever it is stored.
-bool entry_table_pays(int64_t rows, int64_t cols) { return entry_table_size(rows, cols); }
+bool entry_table_pays(int64_t rows, int64_t cols) {
+  constexpr int64_t kLeast = (int64_t)1 << 19;
+  return rows > 0 && cols > 0 && rows >= (kLeast + cols - 1) / cols;
+}
 
 bool entry_table_applies(const bk_opts& o, bk_dtype out_t, double sigma2, double beta, double nu) {
   return o.d_counters == nullptr && o.window != BK_WIN_FIXED && o.series_below == 0.0 &&

@@ -112,13 +112,6 @@ __host__ __device__ inline bool tab_domain(bool f32, double sigma2, double beta,
          sigma2 <= (f32 ? kTabMax32 : 1e20);
 }
 
-// Whether a matrix of rows x cols entries is worth a table (see
-// entry_table_pays).
-__host__ __device__ inline bool entry_table_size(int64_t rows, int64_t cols) {
-  constexpr int64_t kLeast = (int64_t)1 << 19;
-  return rows > 0 && cols > 0 && rows >= (kLeast + cols - 1) / cols;
-}
-
 // One instance of a batch: its descriptor, checked, and its constants.
 struct BatchInstance {
   const double* locs;
@@ -489,12 +482,6 @@ __device__ __forceinline__ unsigned long long mulhi63(unsigned long long a, unsi
   unsigned long long t = (unsigned long long)al * uh;
   t = (unsigned long long)ah * ul + t;
   return (unsigned long long)ah * uh + (t >> 32);
-}
-
-__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
-  long long r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
-  return r;
 }
 
 // Coordinates.  A tile's coordinates are held relative to its first row's point.

@@ -54,6 +54,12 @@ __device__ __forceinline__ float f32_trunc(double v) {
   const unsigned r = (e < -126) ? sign : (e > 127) ? big : (sign | ((unsigned)(e + 127) << 23) | mant);
   return __uint_as_float(r);
 }
+// a b + c, 32 x 32 + 64 bits.
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
 // A float as a double by integer operations only (exact for every input:
 // subnormals are normalised, infinities and NaN payloads kept), so that no
 // conversion is issued on the FP64 pipe.
