@@ -1405,7 +1405,12 @@ __device__ __forceinline__ NodeSum3C node_sum3_cosh(float t0f, float hq, int cou
     D0 = __hiloint2double(__double2hiint(xh) + (1 << 20), __double2loint(xh));
     D1 = xh * c;
   }
-  const unsigned long long Rq = fix64_unit(decay_step(nu, H, tab));
+  // Near nu = 0 the sum of dK/dnu lives on 1 - W, and r's own rounding (2^-54) would
+  // be as large as what was lost before by rounding W: there 1 - r from its series.
+  const double z = 2.0 * nu * H;
+  const unsigned long long Rq =
+      bits_le(z, 0x1p-12) ? ~fix64_unit(z * fma(z, fma(z, fma(z, -1.0 / 24.0, 1.0 / 6.0), -0.5), 1.0))
+                          : fix64_unit(decay_step(nu, H, tab));
   // nu t_j on the nodes of the recurrence with c (rms errors 8e-14 -> 3e-14)
   const double Hs = step_idx >= 0 ? H + widen_f(kCoshShift[step_idx]) : H;
   const long long Gs = __double2ll_rn(nu * Hs * kExpScale40);
