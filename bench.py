@@ -63,7 +63,7 @@ def parse():
     p.add_argument("--pairs", type=int, default=100_000_000,
                    help="K_nu pairs of the learned-window evaluation workload")
     p.add_argument("--profile-case", choices=["plain", "plain_nus", "plain_eval", "fp32", "learned",
-                                              "learned_eval", "batched", "fp32_forms", "train"],
+                                              "learned_eval", "batched", "fp32_forms", "loglik", "train"],
                    default=None,
                    help="run --warmup launches plus one launch of one kernel on a small case "
                         "(for profiler captures) and exit without a JSON line")
@@ -697,6 +697,15 @@ def profile_case(args):
         beta, nu = (0.1, 0.5) if c == "plain" else ((0.05, 2.876) if c == "fp32" else (0.1, 1.7))
         opts = bk.make_opts(learned=net) if c == "learned" else None
         run = lambda: bk.bk_matern_tile(L, 1.0, beta, nu, out=out, opts=opts)
+    elif c == "loglik":  # one likelihood of n = 6,000: 94 panels, 93 updates a pass
+        n = 6000
+        L = torch.as_tensor(inputs.morton_sorted(inputs.jittered_grid(n, seed=4)), device=dev)
+        out = torch.empty((n, n), dtype=torch.float64, device=dev)
+        z = torch.ones(n, dtype=torch.float64, device=dev)
+
+        def run():
+            bk.bk_matern_tile(L, 1.0, BETA, 0.5, out=out)
+            bk.bk_gaussian_loglik(out, z)
     elif c == "plain_eval":
         # the plain FP64 bare evaluation on 10^7 pairs of the 100,000-pair
         # workload's distribution (x log-uniform in [1e-3, 140], nu in [0.05,
@@ -724,10 +733,10 @@ def profile_case(args):
 
 
 def profile_plain_nus(bk, inputs, dev):
-    """The plain FP64 tile writer on the n = 6,000 case for nu = 0.5, 1.5 and
-    2.3: one launch each with the counters (nodes per entry, printed as one
-    JSON line), then one launch each without them, the three launches an FP64
-    instruction-count capture takes (-k regex:matern_sym -s 3 -c 3)."""
+    """The plain FP64 form entry by entry on the n = 6,000 case for nu = 0.5, 1.5
+    and 2.3: one launch each with the counters (nodes per entry, printed as one
+    JSON line), which an FP64 instruction-count capture takes (-k regex:matern_sym
+    -c 3)."""
     import torch
     n = 6000
     L = torch.as_tensor(inputs.morton_sorted(inputs.jittered_grid(n, seed=4)), device=dev)
@@ -740,8 +749,6 @@ def profile_plain_nus(bk, inputs, dev):
         res[str(nu)] = {"entries": n * n, "evals": int(c[bk.BK_CTR_EVALS]),
                         "nodes_per_eval": float(c[bk.BK_CTR_NODES]) / max(1, int(c[bk.BK_CTR_EVALS])),
                         "fallback": int(c[bk.BK_CTR_FALLBACK])}
-    for nu in NUS:
-        bk.bk_matern_tile(L, 1.0, BETA, nu, out=out)
     torch.cuda.synchronize()
     print(json.dumps(res))
 
