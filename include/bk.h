@@ -229,11 +229,16 @@ bk_status bk_matern_tile2(const double* locs1, int64_t m, const double* locs2, i
  * cols) bytes, matrices of at least 2^19 entries are written from a table of
  * that function that the call first builds in the workspace, on `stream`, from
  * the integral of Sec. IV-B (piecewise polynomials, errors below those of the
- * per-entry quadrature; entries with x = r / beta outside about [2.5e-4, 90]
- * and coincident pairs are evaluated directly).  The table is used for the
+ * per-entry quadrature).  It covers x = r / beta from about 2.4e-3 to 110 (the
+ * binades' ends, which depend on beta, are up to sqrt(2) off); for nu < 1/2 the
+ * lower end rises with the span of a 64 x 64 tile's points, to 1.4 at most, and tiles
+ * that span 512 beta (64 in FP32) do not use it.  Other pairs are evaluated directly,
+ * by the searched window of the table's precision; coincident ones are sigma^2, and
+ * pairs beyond the table whose value underflows the output type are zero.  The table is used for the
  * searched and learned windows of either compute type, 0.02 <= nu <= 10,
- * 1e-8 <= beta <= 1e8, 1e-20 <= sigma^2 <= 1e20, and without counters,
- * search_f64 and series_below (options that ask for the per-entry evaluation).
+ * 1e-8 <= beta <= 1e8, 1e-20 <= sigma^2 <= 1e20 (2^50 with FP32 arithmetic into FP32
+ * matrices), and without counters, search_f64 and series_below (options that ask
+ * for the per-entry evaluation).
  * With at least BK_COSH_TABLE_LEN doubles the plain form otherwise keeps its
  * e^{-2 nu h} table there (as bk_opts.d_cosh_table); d_work == NULL, or less, is
  * bk_matern_tile_ex or bk_matern_tile2.  No call allocates.
@@ -302,6 +307,11 @@ bk_status bk_morton_order(const double* locs, int64_t n, int64_t* perm);
  * list and that counter; the call itself allocates nothing and does not
  * synchronise, so it can be captured in a CUDA graph.  Calls that use the
  * same plan must not overlap on the GPU (they share the counter).
+ * A plan whose larger instances together are worth it also owns an entry table for
+ * each instance (at most 1 GiB; see bk_matern_tile_ws, same options and
+ * parameters).  Its calls are three launches: the tables, the tiles of the instances
+ * of n >= 256 (480 with FP32 arithmetic into FP64 matrices) whose parameters the
+ * tables cover, whatever the window, and the other instances in the plan's own form.
  */
 typedef struct {
   const double* locs; /* device, 2n doubles (SoA) */
@@ -315,12 +325,13 @@ typedef struct bk_plan bk_plan;
 
 /* sizes: HOST array of `count` instance sizes.  dtype: output dtype of every
    instance; opts (may be NULL) selects the form (default: compute = dtype).
-   Allocates the plan's device work list; picks a launch shape from the
-   autotune cache when one exists for this GPU, dtype, form and size bucket. */
+   Allocates the plan's device work list (and its tables); picks a launch shape from
+   the autotune cache when one exists for this GPU, dtype, form and size bucket. */
 bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t count,
                                  bk_dtype dtype, const bk_opts* opts);
 bk_status bk_batched_plan_destroy(bk_plan* plan);
-/* Reports the work list size and the launch shape (any output may be NULL). */
+/* Reports the work list size (tiles of 32 x 32, all instances) and the launch shape
+   (any output may be NULL). */
 bk_status bk_batched_plan_info(const bk_plan* plan, int64_t* total_tiles, int* warps,
                                int* ctas_per_sm, int* chunk, int* tuned);
 /* Times launch shapes (warps per CTA, CTAs per SM, tiles per grab) on the

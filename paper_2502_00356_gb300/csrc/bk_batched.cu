@@ -5,7 +5,8 @@
 // every instance: CTAs take tiles from a device counter, so instances of any
 // size share the machine without a launch per matrix.  The plan owns the
 // work list (tile prefix sums per instance) and the counter; the hot call is
-// one memset + one launch, both capturable in a CUDA graph.
+// one memset + one launch, or with entry tables (bk_entry_table.cu) three launches,
+// all capturable in a CUDA graph.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -27,13 +27,14 @@ __global__ void __launch_bounds__(kTabThreads) entry_table_kernel(
 }
 
 // One 64 x 64 tile per block of 256 threads; lane i of warp w evaluates rows
-// i and i + 32 against columns 8 w .. 8 w + 7.  Block (I, J) is stored straight
+// i and i + 32 against columns w, w + 8, w + 16, ...  Block (I, J) is stored straight
 // from registers (a warp writes 32 consecutive rows of one column); for a
 // symmetric matrix the tile also goes through shared memory to block (J, I).
 // col_base as in matern_sym_kernel, in tiles of 64.  FP32 entries wait on their
 // record's load more than on anything else (n = 40,000: 4 blocks an SM 1,883 us,
 // 6 1,699, 8 1,988, spilling a few registers outside the loop); FP64 entries
-// do not gain from more (n = 20,000: 3 blocks 1,139, 4 1,079, 5 1,081, 6 1,142).
+// do not gain from more (n = 20,000: 3 blocks 1,139, 4 1,079, 5 1,081, 6 1,142; now
+// 1,673 and 1,040).
 template <bool F32, typename OutT, bool kSym>
 __global__ void __launch_bounds__(256, F32 ? 6 : 4) matern_table_kernel(
     const unsigned char* table, const double* __restrict__ locs1, int64_t m,

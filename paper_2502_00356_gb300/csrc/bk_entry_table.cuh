@@ -27,8 +27,9 @@
 // with K's ratios for nu = 0.02 to 10).  FP32: one or two bits less and a cubic
 // (an economised quartic; 1e-8 at worst, for nu = 0.02, else below 5e-9).
 // Few and wide intervals mean few cache lines for a warp's record loads, which
-// bound the writers.  Binades with x^2 in [2^-18, 2^13) are covered (x from
-// 2.8e-3 to 90); entries outside take the direct evaluation, or are zero.
+// bound the writers.  Binades with x^2 from f 2^-18 to f 2^13, f in [1, 2) by beta
+// (tab_scale), are covered: x from 2.0e-3 .. 2.8e-3 to 90 .. 128.  Entries outside
+// take the direct evaluation, or are zero.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -623,7 +624,7 @@ __device__ __forceinline__ bool tab_stage(TabPoints<F32>& sm, const double* __re
 
 // M between the points a and b; NaN when they lie outside the table.  FP64: about
 // 95 instructions, 16 of them wide products of 8 cycles a warp and scheduler; with
-// the FP64 pipe's distance n = 20,000 took 1,616 us, now 1,054 (bytes: 480).
+// the FP64 pipe's distance n = 20,000 took 1,616 us, now 1,040 (bytes: 480).
 __device__ __forceinline__ double tab_entry(const unsigned char* table, const int* s_oct,
                                             const int4& p, const int4& q) {
   const int dx = q.x - p.x, lx = q.y - p.y, dy = q.z - p.z, ly = q.w - p.w;

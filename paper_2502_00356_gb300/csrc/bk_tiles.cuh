@@ -497,7 +497,7 @@ int grid_for(int64_t work_items, int per_sm);
 // (block_range); or, where that gives every SM fewer runs of 32 pairs, the fewest
 // blocks of up to eight warps that hold all pairs at once: 100,000 pairs are 21
 // runs an SM in three blocks of seven warps, where blocks of 128 put 24 on some
-// SMs (38.5 -> 34.6 us).  Blocks of fewer than four warps would sort too few pairs
+// SMs (34.9 -> 32.7 us).  Blocks of fewer than four warps would sort too few pairs
 // (1,000 evaluations in blocks of 64 took 27.4 us, in blocks of 128 25.5).
 struct WaveShape {
   int grid, block;
