@@ -248,7 +248,7 @@ __device__ __forceinline__ void tab_scan(float (*s_box)[4], const double* __rest
   for (int set = 0; set < 2; ++set) {
     const double* const l = set ? locs2 : locs1;
     const int64_t len = set ? n : m;
-    if (set && locs2 == locs1) break;
+    if (set && locs2 == locs1 && n == m) break;
 #pragma unroll 4
     for (int64_t i = threadIdx.x % kTabScanThreads; i < len; i += kTabScanThreads) {
 #pragma unroll

@@ -103,3 +103,19 @@ def test_fp32_tables_hold_values_up_to_2_to_the_50(dev, sigma2, table):
     torch.cuda.synchronize()
     assert bool((work != 0xA5).any()) == table
     assert bool(((out.double() - want).abs() <= 2e-6 * want).all())
+
+
+def test_two_sets_that_start_at_the_same_address(dev):
+    """m and n points from one buffer: x and y of the second set are other parts of
+    it, and its distances reach further than the first set's."""
+    m, n = 1000, 700
+    g = torch.Generator(device=dev).manual_seed(3)
+    buf = torch.rand(2 * m, generator=g, dtype=torch.float64, device=dev)
+    buf[m:] += 10.0  # the first set lies in [0, 1] x [10, 11], the second's y also in [0, 1]
+    out = torch.empty((n, m), dtype=torch.float64, device=dev)
+    work = torch.zeros(bk.lib().bk_matern_workspace(m, n), dtype=torch.uint8, device=dev)
+    assert bk.lib().bk_matern_tile2_ws(buf.data_ptr(), m, buf.data_ptr(), n, 1.0, 1.0, 1.5, out.data_ptr(), m, bk.BK_F64, None,
+                                       work.data_ptr(), work.numel(), torch.cuda.current_stream().cuda_stream or None) == bk.BK_OK
+    want = bk.bk_matern_tile2(buf.view(2, m), buf[:2 * n].view(2, n).clone(), 1.0, 1.0, 1.5, opts=direct())
+    torch.cuda.synchronize()
+    assert bool(((out - want).abs() <= 4e-13 * want).all())
