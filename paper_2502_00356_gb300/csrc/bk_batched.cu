@@ -142,6 +142,8 @@ struct bk_plan {
   // and their offsets, the instances' constants, their tables, and a flag for each
   // instance that the per-entry kernel takes
   int64_t table_tiles;
+  int with_table;                  // instances that may have a table, first in d_order
+  int* d_order;
   int64_t* d_table_prefix;
   void* d_inst;
   void* d_tables;
@@ -213,7 +215,7 @@ bool plan_table_f32(const bk_plan* p) { return p->opts.compute == BK_F32 && p->d
 cudaError_t launch_batched(const bk_plan* p, const bk_matern_desc* d, int64_t limit, int warps,
                            int ctas_per_sm, int chunk, cudaStream_t s) {
   if (p->d_tables != nullptr) {
-    const BatchTable b{p->count, p->d_table_prefix, p->d_sizes, p->d_next, p->d_direct, p->d_inst, p->d_tables,
+    const BatchTable b{p->count, p->with_table, p->d_order, p->d_table_prefix, p->d_sizes, p->d_next, p->d_direct, p->d_inst, p->d_tables,
                        p->opts.compute == BK_F64};
     const int64_t tiles = limit < p->total_tiles
                               ? std::max<int64_t>(1, (int64_t)((double)p->table_tiles * limit / p->total_tiles))
@@ -353,14 +355,16 @@ void free_tables(bk_plan* p) {
   cudaFree(p->d_inst);
   cudaFree(p->d_direct);
   cudaFree(p->d_tables);
+  cudaFree(p->d_order);
+  p->d_order = nullptr;
   p->d_table_prefix = nullptr;
   p->d_inst = p->d_tables = nullptr;
   p->d_direct = nullptr;
 }
 
 // Whether an instance of a plan with tables is worth one.  Many tables are built
-// side by side, in 2.4 us each (FP32 1.05): 300 instances of n = 300 took 741 us with
-// them and 2,263 without, in FP32 321 and 859, with the learned window 321 and 753;
+// side by side, in 2.4 us each (FP32 1.1): 300 instances of n = 300 take 763 us with
+// them and 2,263 without, in FP32 347 and 859, with the learned window 347 and 753;
 // 20 of them 88 and 176, 49 and 54, 49 and 62.  FP32 arithmetic into FP64 matrices
 // needs FP64 tables: 20 of n = 300 88 us with, 71 without (learned 65), 40 of n = 400
 // 200 and 219 (195), 40 of n = 500 212 and 310 (279).
@@ -368,24 +372,23 @@ bool batch_instance_pays(int64_t n, const bk_opts& o, bk_dtype out_t) {
   return n >= (o.compute == BK_F32 && out_t == BK_F64 ? 480 : 256);
 }
 // Whether a batch is worth tables: by the entries of the instances that are worth one,
-// as tables cost the call about 40 us (FP32 30).  Batches of such instances alone are
-// bound by one entry's latency without them, and gain early: one matrix of n = 750
-// 42 us with tables, 60 without (FP64), 31, 24 (FP32), 30, 21 (learned); of n = 1,000
-// 42, 92; 32, 33; 32, 30; FP32 arithmetic into FP64, n = 1,000 42, 34, n = 1,250 44,
-// 44.  Beside smaller instances, which keep the GPU busy and then take a launch of their
-// own, the larger ones' entries must be worth the tables by themselves (n = 900
-// beside 200 of n = 100: 390 us with tables, 342 without; FP32 164, 130).
+// in units of 2^19, as tables cost the call about 40 us (FP32 30).  Times in us with
+// tables and without: one matrix of n = 750 42, 60 (FP64), 31, 24 (FP32), 30, 21
+// (learned); of n = 1,000 42, 92; 32, 33; 32, 30; FP32 arithmetic into FP64, n = 1,000
+// 42, 34, n = 1,250 44, 44.  Beside smaller instances, which take a launch of their own
+// then: n = 900 beside one of 30 73, 86 (FP64); n = 1,100 beside one of 100 82, 108;
+// 48, 42; 47, 40; two of n = 900 81, 137; 49, 51; 48, 48; n = 2,000 beside 200 of 100
+// 349, 519; 155, 185; 143, 167; FP32 into FP64 n = 1,500 beside one of 200 61, 59, three
+// of n = 1,000 65, 82.
 bool batch_pays(const int64_t* sizes, int32_t count, const bk_opts& o, bk_dtype out_t) {
-  constexpr double kUnit = 524288.0;  // 2^19 entries
-  const bool f32 = o.compute == BK_F32;
-  const double least = f32 ? (out_t == BK_F64 ? 3.0 * kUnit : 2.0 * kUnit) : kUnit;
   double entries = 0.0;
   bool smaller = false;
   for (int32_t k = 0; k < count; ++k) {
     if (batch_instance_pays(sizes[k], o, out_t)) entries += (double)sizes[k] * (double)sizes[k];
     else smaller = smaller || sizes[k] > 0;
   }
-  return entries >= (smaller ? (f32 ? 6.0 : 3.0) : 1.0) * least;
+  const int least = o.compute == BK_F64 ? 1 : out_t == BK_F32 ? (smaller ? 3 : 2) : (smaller ? 5 : 3);
+  return entries >= 524288.0 * least;
 }
 
 std::string make_key(const bk_plan* p) {
@@ -426,6 +429,7 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   for (int32_t k = 0; k < count; ++k)
     if (sizes[k] < 0) return set_error(BK_ERR_INVALID_ARG, "sizes[%d] < 0", (int)k);
   std::vector<int64_t> prefix((size_t)count + 1, 0), table_prefix((size_t)count + 1, 0);
+  std::vector<int> order;
   // Entry tables (bk_entry_table.cuh) for the forms that have them, where the batch
   // is worth them and they fit 1 GiB.  The parameters are only known at each call:
   // instances outside the tables' domain, and those too small for one, are the
@@ -438,7 +442,11 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
     const int64_t nb = (sizes[k] + kTile - 1) / kTile, nt = batch_instance_pays(sizes[k], o, dtype) ? (sizes[k] + 63) / 64 : 0;
     prefix[(size_t)k + 1] = prefix[(size_t)k] + nb * (nb + 1) / 2;
     table_prefix[(size_t)k + 1] = table_prefix[(size_t)k] + nt * (nt + 1) / 2;
+    if (nt > 0) order.push_back(k);
   }
+  const int with_table = (int)order.size();
+  for (int32_t k = 0; k < count; ++k)
+    if (table_prefix[(size_t)k + 1] == table_prefix[(size_t)k]) order.push_back(k);
   bk_plan* p = new bk_plan();
   p->count = count;
   p->dtype = dtype;
@@ -449,6 +457,8 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
   p->d_next = nullptr;
   p->d_wnu = nullptr;
   p->table_tiles = table_prefix.back();
+  p->with_table = with_table;
+  p->d_order = nullptr;
   p->d_table_prefix = nullptr;
   p->d_inst = nullptr;
   p->d_tables = nullptr;
@@ -471,11 +481,14 @@ bk_status bk_batched_plan_create(bk_plan** plan, const int64_t* sizes, int32_t c
     if (cudaMalloc((void**)&p->d_table_prefix, offsets) != cudaSuccess ||
         cudaMalloc(&p->d_inst, (size_t)count * batched_instance_bytes()) != cudaSuccess ||
         cudaMalloc((void**)&p->d_direct, (size_t)count * sizeof(int)) != cudaSuccess ||
+        cudaMalloc((void**)&p->d_order, (size_t)count * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&p->d_tables, table_bytes) != cudaSuccess) {
       (void)cudaGetLastError();  // without them the per-entry kernel takes every instance
       free_tables(p);
     } else {
       e = cudaMemcpy(p->d_table_prefix, table_prefix.data(), offsets, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess)
+        e = cudaMemcpy(p->d_order, order.data(), (size_t)count * sizeof(int), cudaMemcpyHostToDevice);
     }
   }
   // per-instance tables of e^{-2 nu h} for the searched-window FP64 forms

@@ -75,6 +75,8 @@ bool entry_table_applies(const bk_opts& o, bk_dtype out_t, double sigma2, double
 // without a table, whose e^{-2 nu h} then stand in place of the table (decay).
 struct BatchTable {
   int count;
+  int with_table;    // instances that may have one
+  const int* order;  // all instances, those first
   const int64_t* prefix;
   const int64_t* sizes;
   unsigned long long* next;

@@ -81,11 +81,12 @@ def test_instances_without_a_table_keep_their_form(dev, forms, form, dtype):
 
 
 @pytest.mark.parametrize("form,dtype,sizes,table", [
-    ("f64", torch.float64, [725], True), ("f64", torch.float64, [700], False), ("f64", torch.float64, [900, 100], False),
-    ("f64", torch.float64, [900, 900, 100], True), ("f32", torch.float32, [900], False), ("f32", torch.float32, [1024], True),
-    ("learned", torch.float32, [1000], False), ("learned", torch.float32, [400] * 8, True), ("learned", torch.float32, [1500, 200], False),
-    ("learned", torch.float32, [2600, 200], True), ("learned", torch.float64, [1200], False), ("f32", torch.float64, [400] * 40, False),
-    ("f32", torch.float64, [1300], True)])
+    ("f64", torch.float64, [725], True), ("f64", torch.float64, [700], False), ("f64", torch.float64, [900, 100], True),
+    ("f64", torch.float64, [700, 100, 20], False), ("f32", torch.float32, [900], False), ("f32", torch.float32, [1024], True),
+    ("learned", torch.float32, [1000], False), ("learned", torch.float32, [400] * 8, True), ("learned", torch.float32, [1250, 200], False),
+    ("learned", torch.float32, [1260, 200], True), ("learned", torch.float64, [1200], False), ("f32", torch.float64, [400] * 40, False),
+    ("f32", torch.float64, [1300], True), ("f32", torch.float64, [1600, 300], False),
+    ("f32", torch.float64, [1650, 300], True)])
 def test_which_batches_have_tables(dev, forms, form, dtype, sizes, table):
     """By the entries that a table serves; the plan's size is that of its tiles of 32."""
     opts = forms[form]
